@@ -203,6 +203,7 @@ rs_status rs_resize_normalize(const void* src, const rs_layout* in, void* dst, c
     if (li.kind != 0 || (in->C > 1 && lo.kind != 1) || in->N != out->N || in->C != out->C) return RS_ERR_INVALID_ARG;
     NormOut no;
     no.c_stride = out->c_stride;
+    no.dtype = out_dtype;
     for (int c = 0; c < 4; ++c) {
         no.scale[c] = 1.0f;
         no.bias[c] = 0.0f;
@@ -241,6 +242,12 @@ rs_status rs_resize_normalize(const void* src, const rs_layout* in, void* dst, c
         }
     }
     if (!ok) return o.tile_h ? RS_ERR_INVALID_ARG : RS_ERR_UNSUPPORTED;
+    // grey and RGB sources, at most two source pixels per output pixel along
+    // x: the form that reads the source in place
+    WinCfg raw = c;
+    raw.chunk = o.tile_h;
+    if (!win_is_x2(g) && (g.C == 1 || g.C == 3) && win_raw_default(g, method, DT_U8, win_raw_threads(g.Wo, 128), 256, raw))
+        return cuda_status(launch_win_raw_norm(g, method, src, dst, raw, no, static_cast<cudaStream_t>(stream)));
     return cuda_status(launch_win_norm(g, method, out_dtype, src, dst, c, no, static_cast<cudaStream_t>(stream)));
 }
 

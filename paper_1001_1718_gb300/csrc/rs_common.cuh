@@ -20,31 +20,37 @@ namespace rs {
 //   asymmetric:    num = j n,            den = m
 //   half-pixel:    num = (2j + 1) n - m, den = 2 m
 //   align-corners: num = j (n - 1),      den = m - 1  (num = 0, den = 1 if m = 1)
-// i0 = floor(x) and t = (num - i0 den) / den (Eqs. 2-4). The quotient is
-// estimated in FP32 (error < 1 for |num| < 2^34 and den <= 2^17) and then
-// corrected in exact 64-bit integer arithmetic, so i0 is exact and t takes a
-// single rounding (the remainder and den are exact FP32 integers).
+// i0 = floor(x) and t = (num - i0 den) / den (Eqs. 2-4). With num = j step +
+// first, the quotient is estimated in FP32 and then corrected in exact
+// integer arithmetic, so i0 is exact and t takes a single rounding (the
+// remainder and den are exact FP32 integers). All of it in 32 bits: j, step,
+// first and den are below 2^17 and exact in FP32, the estimate's relative
+// error is below 2^-21 and the quotient below 2^16 in magnitude, so it is
+// off by less than 1; the remainder before the correction lies in (-den, 2 den),
+// so its low 32 bits (wrapping products) hold it. (In 64-bit integers a map
+// cost ~100 instructions, a tenth of the uint8 window kernel's at bands of
+// 81 rows.)
 // ---------------------------------------------------------------------------
 
-__device__ __forceinline__ int floor_div_exact(int64_t num, int64_t den, int64_t& rem)
+__device__ __forceinline__ int floor_ratio(int j, int step, int first, int den, int& rem)
 {
-    int64_t q = (int64_t)floorf((float)num / (float)den);
-    int64_t r = num - q * den;
+    int q = __float2int_rd(__fdividef(fmaf((float)j, (float)step, (float)first), (float)den));
+    int r = (int)((uint32_t)j * (uint32_t)step + (uint32_t)first - (uint32_t)q * (uint32_t)den);
     if (r < 0) { q -= 1; r += den; }
     else if (r >= den) { q += 1; r -= den; }
     rem = r;
-    return (int)q;
+    return q;
 }
 
 __device__ __forceinline__ void axis_map(int j, int n, int m, int coord, int& i0, float& t)
 {
-    int64_t num, den;
-    if (coord == COORD_ASYMMETRIC) { num = (int64_t)j * n; den = m; }
-    else if (coord == COORD_HALF_PIXEL) { num = (int64_t)(2 * j + 1) * n - m; den = 2 * (int64_t)m; }
-    else if (m > 1) { num = (int64_t)j * (n - 1); den = m - 1; }
-    else { num = 0; den = 1; }
-    int64_t rem;
-    i0 = floor_div_exact(num, den, rem);
+    int step, first, den;
+    if (coord == COORD_ASYMMETRIC) { step = n; first = 0; den = m; }
+    else if (coord == COORD_HALF_PIXEL) { step = 2 * n; first = n - m; den = 2 * m; }
+    else if (m > 1) { step = n - 1; first = 0; den = m - 1; }
+    else { step = 0; first = 0; den = 1; }
+    int rem;
+    i0 = floor_ratio(j, step, first, den, rem);
     t = __fdiv_rn((float)rem, (float)den);
 }
 
@@ -52,11 +58,11 @@ __device__ __forceinline__ void axis_map(int j, int n, int m, int coord, int& i0
 // align-corners).
 __device__ __forceinline__ int nearest_index(int j, int n, int m, int coord)
 {
-    int64_t rem;
-    if (coord == COORD_ASYMMETRIC) return floor_div_exact((int64_t)j * n, m, rem);
-    if (coord == COORD_HALF_PIXEL) return floor_div_exact((int64_t)(2 * j + 1) * n, 2 * (int64_t)m, rem);
+    int rem;
+    if (coord == COORD_ASYMMETRIC) return floor_ratio(j, n, 0, m, rem);
+    if (coord == COORD_HALF_PIXEL) return floor_ratio(j, 2 * n, n, 2 * m, rem);
     if (m <= 1) return 0;
-    return floor_div_exact((int64_t)2 * j * (n - 1) + (m - 1), 2 * (int64_t)(m - 1), rem);
+    return floor_ratio(j, 2 * (n - 1), m - 1, 2 * (m - 1), rem);
 }
 
 // Index of the first (unclamped) tap of output j for a KT-tap method:

@@ -109,6 +109,8 @@ struct WinCfg {
     int raw_off;     // byte offset of the raw ring in shared memory
     int aa_method;   // antialias taps: M_BILINEAR / M_BICUBIC (the stretched kernel)
     int strip;       // antialias taps: output pixels per block (at most the kernel's 128 P)
+    int pat;         // uint8 sources read in place (win_raw.cuh): the ratio range + 1 (0: the other forms)
+    int nt;          // ditto: threads per block
     size_t smem;
 };
 
@@ -140,6 +142,7 @@ struct AaVsCfg {
 struct NormOut {
     int64_t c_stride;
     float scale[4], bias[4];
+    int dtype;       // output dtype
 };
 
 int method_taps(int method);
@@ -178,6 +181,18 @@ cudaError_t launch_stream(const Geom& g, int method, int dtype, const void* src,
 int win_pixels(int C, int dtype, bool x2);
 bool win_is_x2(const Geom& g);
 bool win_config(const Geom& g, int method, int dtype, WinCfg& c, bool allow_x2 = true);
+// The form that reads uint8 sources in place (win_raw.cuh): configuration for
+// blocks of nt threads and bands of at most band_cap rows (false where it does
+// not apply: other dtypes, more than two source pixels per output pixel along
+// x), its default (c.chunk 0: 8 staged rows at a time, or 4 where 8 leave no
+// room for four blocks per SM) and launches (band_h 0 = from occupancy and
+// waves).
+bool win_raw_config(const Geom& g, int method, int dtype, int nt, int band_cap, WinCfg& c);
+bool win_raw_default(const Geom& g, int method, int dtype, int nt, int band_cap, WinCfg& c);
+int win_raw_threads(int Wo, int warp_px);
+cudaError_t launch_win_raw(const Geom& g, int method, const void* src, void* dst, WinCfg c, cudaStream_t st);
+cudaError_t launch_win_raw_norm(const Geom& g, int method, const void* src, void* dst, WinCfg c, const NormOut& no,
+                                cudaStream_t st);
 cudaError_t launch_win(const Geom& g, int method, int dtype, const void* src, void* dst, WinCfg c, cudaStream_t st);
 // Antialiased resampling (RS_FLAG_ANTIALIAS) on the general window form:
 // the most taps any output has on either axis (antialias_taps), the tap

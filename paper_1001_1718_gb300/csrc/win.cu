@@ -116,6 +116,7 @@ bool win_config(const Geom& g, int method, int dtype, WinCfg& c, bool allow_x2)
     const bool x2 = allow_x2 && win_is_x2(g);
     const int P = win_pixels(g.C, dtype, x2);
     const int SP = kWinThreads * P;
+    c.pat = 0;
     // source pixels a strip's footprint can span
     const int span_px = tap_span_bound(SP, g.W, g.Wo, KT, g.coord);
     const int per = (span_px * g.C * es + 15) / 16 + 1;   // raw 16-byte blocks per row
@@ -197,6 +198,7 @@ bool win_config_aa(const Geom& g, int method, int dtype, int K, WinCfg& c)
 
 cudaError_t launch_win(const Geom& g, int method, int dtype, const void* src, void* dst, WinCfg c, cudaStream_t st)
 {
+    if (c.pat) return launch_win_raw(g, method, src, dst, c, st);
     const bool x2 = win_is_x2(g);
     void* func = win_kernel(method, dtype, g.C, x2);
     int per_sm = 1;
