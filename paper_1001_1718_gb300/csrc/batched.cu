@@ -26,7 +26,7 @@
 #include <vector>
 
 #include "capi_internal.h"
-#include "win_body.cuh"
+#include "win_raw.cuh"
 #include "tile_body.cuh"
 #include "aa_wide.cuh"
 
@@ -37,11 +37,11 @@ struct BatchImage {
     void* dst;
     int64_t src_pitch, dst_pitch;
     int H, W, Ho, Wo;
-    int C, method, tiles_x, kind;          // tiles_x: items per row of items; kind 0 tile, 1 window, 2 many-tap
+    int C, method, tiles_x, kind;          // tiles_x: items per row of items; kind 0 tile, 1 window, 2 many-tap, 3 window in place
     int tile_w, tile_h, sh_max, swe_max;   // kind 0: tiled-kernel tile
     int chunk, band_h, swe, raw_row, band_cap, pos_cap, tab_off, raw_off;   // kind 1: window config
     int aa, strip;                         // antialias taps: the stretched method (0: point taps), window strip
-    int KX, KY, TH, RG, fw, nr, s_off, pad;   // kind 2: many-tap antialias tiles (AaWideCfg)
+    int KX, KY, TH, RG, fw, nr, s_off, pat;   // kind 3: pat (WinCfg); kind 2: many-tap antialias tiles (AaWideCfg)
 };
 
 // Classes: 0..7 = window (KT 2 / 4) x (C 1..4) with a footprint of at most
@@ -51,8 +51,13 @@ struct BatchImage {
 // occupancy of its whole class. With RS_FLAG_ANTIALIAS (the whole batch)
 // the window classes hold antialias taps, at most K = 4 / 8 per axis in
 // place of KT = 2 / 4, and class 16 the many-tap antialias tiles.
-static constexpr int kClasses = 17;
+// Classes 17..32 = (KT 2 / 4) x (C 1..4) of the uint8 window items that read
+// their source in place (win_raw.cuh): up to one source pixel per output
+// pixel along x, then 25.. up to two (twice the footprint).
+static constexpr int kClasses = 33;
 static constexpr int kTileClass = 16;
+static constexpr int kRawClass = 17;
+static constexpr int kRawThreads = kWinThreads;
 static constexpr size_t kWindowSmallSmem = 72 * 1024;
 static constexpr int kHeavyBand = 32;   // band rows of large-footprint and downscaled window items
 
@@ -65,6 +70,39 @@ __device__ __forceinline__ int find_image(const int64_t* __restrict__ start, int
     }
     return lo;
 }
+
+// A block's walk over its class's items. It starts with item blockIdx.x and
+// then takes the next one nobody has: `next` counts the takers, gridDim.x
+// items ahead of it. Items are sorted costliest first, so the blocks that
+// draw cheap items take more of them and all end together (with a fixed
+// stride the slowest SM worked ~10% longer than the mean). The next item is
+// drawn while the current one runs. Every block draws until it draws past the
+// end, `total` draws in all (the grid is no larger than `total`), and the
+// last one sets the counter back to 0 for the next launch.
+struct ItemQueue {
+    unsigned long long* next;
+    int64_t t, total;
+    unsigned long long drawn;   // thread 0
+
+    __device__ __forceinline__ ItemQueue(unsigned long long* n, int64_t total_) : next(n), t(blockIdx.x), total(total_) { draw(); }
+    __device__ __forceinline__ void draw()
+    {
+        if (threadIdx.x == 0 && t < total) drawn = atomicAdd(next, 1ull);
+    }
+    // every thread of the block, done with the item's shared memory
+    __device__ __forceinline__ void advance()
+    {
+        __shared__ int64_t item;
+        if (threadIdx.x == 0) {
+            if (drawn + 1 == (unsigned long long)total) *next = 0ull;
+            item = (int64_t)drawn + gridDim.x;
+        }
+        __syncthreads();
+        t = item;
+        draw();
+        __syncthreads();   // the next item reuses shared memory (and `item`)
+    }
+};
 
 __device__ __forceinline__ Geom image_geom(const BatchImage& im, int coord, float a)
 {
@@ -85,10 +123,11 @@ __device__ __forceinline__ Geom image_geom(const BatchImage& im, int coord, floa
 template <int KT, int C, typename T, int TM = TAP_POINT>
 __global__ void __launch_bounds__(kWinThreads, 2)
 k_batched_window(const BatchImage* __restrict__ imgs, const int64_t* __restrict__ start, int n, int64_t total,
-                 int coord, float a, unsigned int* fault)
+                 unsigned long long* next, int coord, float a, unsigned int* fault)
 {
     extern __shared__ __align__(16) float sm[];
-    for (int64_t t = blockIdx.x; t < total; t += gridDim.x) {
+    for (ItemQueue q(next, total); q.t < total; q.advance()) {
+        const int64_t t = q.t;
         const int k = find_image(start, n, t);
         const BatchImage im = imgs[k];
         const int64_t local = t - __ldg(start + k);
@@ -112,7 +151,48 @@ k_batched_window(const BatchImage* __restrict__ imgs, const int64_t* __restrict_
         wc.smem = 0;
         win_body<KT, C, T, T, false, TM>(g, static_cast<const T*>(im.src), static_cast<T*>(im.dst), wc,
                                          (int)(local % im.tiles_x), (int)(local / im.tiles_x), sm, fault);
-        __syncthreads();   // the next item reuses shared memory
+    }
+}
+
+// Window items of uint8 sources read in place (kind 3), any ratio range.
+// DOWN: more than one source pixel per output pixel along x.
+template <int KT, int C, bool DOWN>
+__global__ void __launch_bounds__(kRawThreads, 4)
+k_batched_raw(const BatchImage* __restrict__ imgs, const int64_t* __restrict__ start, int n, int64_t total,
+              unsigned long long* next, int coord, float a, unsigned int* fault)
+{
+    extern __shared__ __align__(16) float sm[];
+    for (ItemQueue q(next, total); q.t < total; q.advance()) {
+        const int64_t t = q.t;
+        const int k = find_image(start, n, t);
+        const BatchImage im = imgs[k];
+        const int64_t local = t - __ldg(start + k);
+        if (local < 0 || local >= __ldg(start + k + 1) - __ldg(start + k) || im.kind != 3 || im.C != C || (im.pat == 3) != DOWN) {
+            if (threadIdx.x == 0) report_fault(fault, FAULT_BATCH_INDEX);   // uniform over the block
+            continue;
+        }
+        const Geom g = image_geom(im, coord, a);
+        WinCfg wc;
+        wc.chunk = im.chunk;
+        wc.band_h = im.band_h;
+        wc.waves = 0;
+        wc.swe = 0;
+        wc.raw_row = im.raw_row;
+        wc.band_cap = im.band_cap;
+        wc.pos_cap = im.pos_cap;
+        wc.tab_off = im.tab_off;
+        wc.raw_off = im.raw_off;
+        wc.aa_method = 0;
+        wc.strip = 0;
+        wc.pat = im.pat;
+        wc.nt = kRawThreads;
+        wc.smem = 0;
+        const uint8_t* s = static_cast<const uint8_t*>(im.src);
+        uint8_t* d = static_cast<uint8_t*>(im.dst);
+        const int bx = (int)(local % im.tiles_x), by = (int)(local / im.tiles_x);
+        if constexpr (DOWN) win_body_raw<KT, C, 2, RAW_ANY>(g, s, d, wc, bx, by, sm, fault);
+        else if (im.pat == 1) win_body_raw<KT, C, 0, RAW_ANY>(g, s, d, wc, bx, by, sm, fault);
+        else win_body_raw<KT, C, 1, RAW_ANY>(g, s, d, wc, bx, by, sm, fault);
     }
 }
 
@@ -120,10 +200,11 @@ k_batched_window(const BatchImage* __restrict__ imgs, const int64_t* __restrict_
 template <typename T>
 __global__ void __launch_bounds__(kAwNT)
 k_batched_aa_wide(const BatchImage* __restrict__ imgs, const int64_t* __restrict__ start, int n, int64_t total,
-                  int coord, float a, unsigned int* fault)
+                  unsigned long long* next, int coord, float a, unsigned int* fault)
 {
     extern __shared__ __align__(16) float sm[];
-    for (int64_t t = blockIdx.x; t < total; t += gridDim.x) {
+    for (ItemQueue q(next, total); q.t < total; q.advance()) {
+        const int64_t t = q.t;
         const int k = find_image(start, n, t);
         const BatchImage im = imgs[k];
         const int64_t local = t - __ldg(start + k);
@@ -145,7 +226,6 @@ k_batched_aa_wide(const BatchImage* __restrict__ imgs, const int64_t* __restrict
         case 3: aa_wide_body<3, T, T, false>(g, s, d, c, bx, by, sm, fault, NormOut{}); break;
         default: aa_wide_body<4, T, T, false>(g, s, d, c, bx, by, sm, fault, NormOut{}); break;
         }
-        __syncthreads();   // the next tile reuses shared memory
     }
 }
 
@@ -167,10 +247,11 @@ __device__ __forceinline__ void batch_tile_c(const Geom& g, const BatchImage& im
 template <typename T>
 __global__ void __launch_bounds__(256)
 k_batched(const BatchImage* __restrict__ imgs, const int64_t* __restrict__ start, int n, int64_t total,
-          int coord, float a, unsigned int* fault)
+          unsigned long long* next, int coord, float a, unsigned int* fault)
 {
     extern __shared__ __align__(16) float sm[];
-    for (int64_t t = blockIdx.x; t < total; t += gridDim.x) {
+    for (ItemQueue q(next, total); q.t < total; q.advance()) {
+        const int64_t t = q.t;
         const int k = find_image(start, n, t);
         const BatchImage im = imgs[k];
         const int64_t local = t - __ldg(start + k);
@@ -192,7 +273,6 @@ k_batched(const BatchImage* __restrict__ imgs, const int64_t* __restrict__ start
         case M_BILINEAR: batch_tile_c<2, T>(g, im, cfg, bx, by, sm, fault); break;
         default: batch_tile_c<4, T>(g, im, cfg, bx, by, sm, fault); break;
         }
-        __syncthreads();   // the next tile reuses shared memory
     }
 }
 
@@ -310,6 +390,27 @@ static rs_status prepare_image(const rs_image_desc& x, int dtype, const rs_optio
             wc.chunk = ch;
             // the general window body (the batch has no exact-x2 form: one kernel per class)
             if (!win_config(g, x.method, dtype, wc, false) || wc.smem > (t < 2 ? kWindowSmallSmem : 100 * 1024)) continue;
+            WinCfg raw{};
+            raw.chunk = sh.chunk;
+            // a downscale's output row takes several source rows: shorter bands
+            const int band = x.Ho < x.H ? std::max(std::min(sh.band, kHeavyBand), (int)((int64_t)sh.band * x.Ho / x.H)) : sh.band;
+            if (win_raw_default(g, x.method, dtype, kRawThreads, band, raw)) {   // uint8 read in place
+                im.kind = 3;
+                im.pat = raw.pat;
+                im.chunk = raw.chunk;
+                im.band_h = raw.band_cap;
+                im.raw_row = raw.raw_row;
+                im.band_cap = raw.band_cap;
+                im.pos_cap = raw.pos_cap;
+                im.raw_off = raw.raw_off;
+                im.tab_off = raw.tab_off;
+                const int strip = raw_strip(kRawThreads, raw_overlap(RAW_ANY, 1));
+                im.tiles_x = (int)(((int64_t)x.Wo + strip - 1) / strip);
+                items = (int64_t)im.tiles_x * ((x.Ho + im.band_h - 1) / im.band_h);
+                smem = raw.smem;
+                cls = kRawClass + (raw.pat == 3 ? 8 : 0) + (x.method == RS_BILINEAR ? 0 : 4) + (x.C - 1);
+                return RS_OK;
+            }
             im.kind = 1;
             im.chunk = wc.chunk;
             // A large footprint or a vertical downscale makes each band row
@@ -347,13 +448,13 @@ static rs_status prepare_image(const rs_image_desc& x, int dtype, const rs_optio
 // column), plus a fixed part for the block's prologue.
 static int64_t image_items(const BatchImage& im)
 {
-    const int rows = im.kind == 1 ? im.band_h : im.kind == 2 ? im.TH : im.tile_h;
+    const int rows = im.kind == 1 || im.kind == 3 ? im.band_h : im.kind == 2 ? im.TH : im.tile_h;
     return (int64_t)im.tiles_x * ((im.Ho + rows - 1) / rows);
 }
 
 static double item_cost(const BatchImage& im)
 {
-    const int rows = im.kind == 1 ? im.band_h : im.kind == 2 ? im.TH : im.tile_h;
+    const int rows = im.kind == 1 || im.kind == 3 ? im.band_h : im.kind == 2 ? im.TH : im.tile_h;
     return rows * (1.0 + 0.55 * (double)im.H / (double)im.Ho) + 24.0;
 }
 
@@ -370,8 +471,8 @@ struct BatchLayout {
     int n;
 };
 
-// Fills imgs_out (n entries) and start_out (n + kClasses entries) grouped
-// by class, with no allocation (scratch arrays are caller-provided, n each).
+// Fills imgs_out (n entries) and start_out (n + kClasses prefix entries, then
+// kClasses zero item counters) grouped by class, with no allocation (scratch arrays are caller-provided, n each).
 // Tuning-cache key of a batch: GPU (model, CUDA runtime, SM count), dtype,
 // count, coordinate map and a hash of every descriptor's sizes, channels,
 // method and pitches.
@@ -399,6 +500,19 @@ static std::string batch_key(const rs_image_desc* d, int n, int dtype, const rs_
 // (default 256) and chunk = tile_h (default 0); RS_IMPL_AUTO takes the
 // tuned shape of this batch when the cache has one (`tuned`), else the
 // default window shape. Other kernels have no batched form.
+static constexpr int kBandItems = 4;   // items wanted per resident block slot (of four per SM)
+
+// Default band: enough items for every resident slot to draw a few (the
+// queue evens them out), within 32 rows (a band's tables, first copies and
+// the KT - 1 rows above it cost about ten of its rows) and 256.
+static int default_band(const rs_image_desc* d, int n)
+{
+    int64_t rows = 0;   // strips x output rows
+    for (int k = 0; k < n; ++k) rows += (int64_t)((std::max(d[k].Wo, 1) + 495) / 496) * std::max(d[k].Ho, 1);
+    const int64_t band = rows / ((int64_t)kBandItems * 4 * num_sms());
+    return (int)std::min<int64_t>(kWinMaxBand, std::max<int64_t>(32, (band + 7) / 8 * 8));
+}
+
 static rs_status batch_shape(const rs_image_desc* d, int n, int dtype, const rs_options& o, bool tuned,
                              BatchShape& sh)
 {
@@ -414,7 +528,7 @@ static rs_status batch_shape(const rs_image_desc* d, int n, int dtype, const rs_
         return RS_OK;
     }
     if (o.impl != RS_IMPL_AUTO) return RS_ERR_INVALID_ARG;
-    sh = BatchShape{false, 0, kWinMaxBand};
+    sh = BatchShape{false, 0, default_band(d, n)};
     Tuned t;
     if (tuned && tune_lookup(batch_key(d, n, dtype, o), t)) {
         if (t.impl == RS_IMPL_TILED) sh = BatchShape{true, 0, 0};
@@ -468,6 +582,7 @@ static rs_status batch_layout(const rs_image_desc* d, int n, int dtype, const rs
     for (int c = 0; c < kClasses; ++c) {
         fill[c] = 0;
         start_out[L.prefix[c]] = 0;
+        start_out[n + kClasses + c] = 0;   // item counter
     }
     for (int k = 0; k < n; ++k) {
         const int c = tmp_cls[k];
@@ -534,8 +649,30 @@ static void* class_func_t(int c, bool aa)
     }
 }
 
+template <int KT, int C>
+static void* raw_func_d(bool down)
+{
+    return down ? reinterpret_cast<void*>(&k_batched_raw<KT, C, true>) : reinterpret_cast<void*>(&k_batched_raw<KT, C, false>);
+}
+
+static void* raw_func(int c)
+{
+    const bool down = c - kRawClass >= 8;
+    switch ((c - kRawClass) & 7) {
+    case 0: return raw_func_d<2, 1>(down);
+    case 1: return raw_func_d<2, 2>(down);
+    case 2: return raw_func_d<2, 3>(down);
+    case 3: return raw_func_d<2, 4>(down);
+    case 4: return raw_func_d<4, 1>(down);
+    case 5: return raw_func_d<4, 2>(down);
+    case 6: return raw_func_d<4, 3>(down);
+    default: return raw_func_d<4, 4>(down);
+    }
+}
+
 static void* class_func(int dtype, int c, bool aa)
 {
+    if (c >= kRawClass) return raw_func(c);
     switch (dtype) {
     case DT_U8: return class_func_t<uint8_t>(c, aa);
     case DT_F16: return class_func_t<__half>(c, aa);
@@ -554,6 +691,7 @@ struct ClassLaunch {
     const int64_t* start;
     int n;
     int64_t total;
+    unsigned long long* next;   // the class's item counter (ItemQueue)
     int coord;
     float a;
     unsigned int* fault;
@@ -581,7 +719,7 @@ static cudaError_t class_launches(const BatchLayout& L, int dtype, const rs_opti
         ClassLaunch& cl = out[nl++];
         const bool aa = (o.flags & RS_FLAG_ANTIALIAS) != 0;
         cl.func = class_func(dtype, c, aa);
-        const int threads = c == kTileClass ? (aa ? kAwNT : L.threads) : kWinThreads;
+        const int threads = c == kTileClass ? (aa ? kAwNT : L.threads) : c >= kRawClass ? kRawThreads : kWinThreads;
         int per_sm = 0;
         cudaError_t e = prepare_kernel(cl.func, L.smem[c], threads, &per_sm);
         if (e != cudaSuccess) return e;
@@ -593,6 +731,7 @@ static cudaError_t class_launches(const BatchLayout& L, int dtype, const rs_opti
         cl.start = static_cast<const int64_t*>(start_dev) + L.prefix[c];
         cl.n = L.count[c];
         cl.total = L.total[c];
+        cl.next = static_cast<unsigned long long*>(const_cast<void*>(start_dev)) + L.n + kClasses + c;
         cl.coord = o.coord;
         cl.a = o.cubic_a;
         cl.fault = fault_word();
@@ -604,7 +743,7 @@ static cudaError_t launch_classes(ClassLaunch* cls, int nl, cudaStream_t st)
 {
     for (int i = 0; i < nl; ++i) {
         ClassLaunch& c = cls[i];
-        void* args[] = {&c.imgs, &c.start, &c.n, &c.total, &c.coord, &c.a, &c.fault};
+        void* args[] = {&c.imgs, &c.start, &c.n, &c.total, &c.next, &c.coord, &c.a, &c.fault};
         cudaError_t e = cudaLaunchKernel(c.func, c.grid, c.block, args, c.smem, st);
         if (e == cudaSuccess) e = cudaGetLastError();
         if (e != cudaSuccess) return e;
@@ -624,7 +763,7 @@ static rs_status batch_prepare(const rs_image_desc* d, int n, int dtype, const r
 {
     if (!d || n < 1 || n > (1 << 20)) return RS_ERR_INVALID_ARG;
     P.imgs.resize(n);
-    P.start.assign((size_t)n + kClasses, 0);
+    P.start.assign((size_t)n + 2 * kClasses, 0);   // prefixes, then the classes' item counters
     std::vector<BatchImage> tmp(n);
     std::vector<int> cls(n);
     std::vector<int64_t> items(n);
@@ -672,14 +811,14 @@ static rs_status check_ws(const BatchPlanHost& P, void* ws, size_t bytes)
 // device current) and passed to the kernel like any other pointer.
 static constexpr int kNoAllocMaxImages = 4096;
 static constexpr size_t kNoAllocImgBytes = ((sizeof(BatchImage) * kNoAllocMaxImages + 255) / 256) * 256;
-static constexpr size_t kNoAllocBytes = kNoAllocImgBytes + sizeof(int64_t) * (kNoAllocMaxImages + kClasses);
+static constexpr size_t kNoAllocBytes = kNoAllocImgBytes + sizeof(int64_t) * (kNoAllocMaxImages + 2 * kClasses);
 static __device__ __align__(256) unsigned char g_batch_scratch[kNoAllocBytes];
 
 static constexpr int kNoAllocMaxDevices = 64;
 static std::mutex g_noalloc_mu;                               // guards everything below
 static void* g_noalloc_dev[kNoAllocMaxDevices];               // device address per device
 static BatchImage g_noalloc_imgs[kNoAllocMaxImages];           // host staging (no heap use)
-static int64_t g_noalloc_start[kNoAllocMaxImages + kClasses];
+static int64_t g_noalloc_start[kNoAllocMaxImages + 2 * kClasses];   // prefixes, then item counters (0)
 static BatchImage g_noalloc_tmp[kNoAllocMaxImages];
 static int g_noalloc_cls[kNoAllocMaxImages];
 static int64_t g_noalloc_items[kNoAllocMaxImages];
@@ -723,7 +862,7 @@ extern "C" rs_status rs_resize_batched_noalloc(const rs_image_desc* d, int n, rs
     // so the staging arrays may be refilled by the next call.
     e = cudaMemcpyAsync(scratch, g_noalloc_imgs, sizeof(BatchImage) * (size_t)n, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess)
-        e = cudaMemcpyAsync(scratch + kNoAllocImgBytes, g_noalloc_start, sizeof(int64_t) * (size_t)(n + kClasses),
+        e = cudaMemcpyAsync(scratch + kNoAllocImgBytes, g_noalloc_start, sizeof(int64_t) * (size_t)(n + 2 * kClasses),
                             cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) return cuda_status(e);
     ClassLaunch cls[kClasses];
@@ -801,7 +940,7 @@ rs_status rs_batched_plan_create(const rs_image_desc* d, int n, rs_dtype dtype, 
     // class launches may run concurrently.
     for (int i = 0; i < nl && e == cudaSuccess; ++i) {
         ClassLaunch& c = cls[i];
-        void* args[] = {&c.imgs, &c.start, &c.n, &c.total, &c.coord, &c.a, &c.fault};
+        void* args[] = {&c.imgs, &c.start, &c.n, &c.total, &c.next, &c.coord, &c.a, &c.fault};
         cudaKernelNodeParams kp;
         std::memset(&kp, 0, sizeof kp);
         kp.func = c.func;
@@ -857,7 +996,9 @@ rs_status rs_autotune_batched(const rs_image_desc* d, int n, rs_dtype dtype, voi
         int impl, band, chunk;
     };
     // The default shape first, then band heights x chunk heights, then tiles.
-    const Cand cands[] = {{RS_IMPL_WINDOW, 256, 0}, {RS_IMPL_WINDOW, 128, 0}, {RS_IMPL_WINDOW, 64, 0},
+    if (!d || n < 1) return RS_ERR_INVALID_ARG;
+    const Cand cands[] = {{RS_IMPL_WINDOW, default_band(d, n), 0},
+                          {RS_IMPL_WINDOW, 256, 0}, {RS_IMPL_WINDOW, 128, 0}, {RS_IMPL_WINDOW, 64, 0},
                           {RS_IMPL_WINDOW, 32, 0},  {RS_IMPL_WINDOW, 256, 4}, {RS_IMPL_WINDOW, 128, 4},
                           {RS_IMPL_WINDOW, 64, 4},  {RS_IMPL_TILED, 0, 0}};
     cudaStream_t st = static_cast<cudaStream_t>(stream);
