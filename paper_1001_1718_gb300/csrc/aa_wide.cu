@@ -4,7 +4,8 @@
 // ratio), for every storage dtype and for the fused pre-process's
 // normalised planar output, and their host configuration.
 #include <algorithm>
-#include <vector>
+#include <cmath>
+#include <type_traits>
 
 #include "capi_internal.h"
 #include "aa_wide.cuh"
@@ -24,7 +25,7 @@ k_aa_wide(const Geom g, const T* __restrict__ src, TO* __restrict__ dst, const A
 }
 
 template <int C, typename T, typename TO, bool NORM, int NA>
-__global__ void __launch_bounds__(kVsNT, 3)
+__global__ void __launch_bounds__(kVsNT, 5)
 k_aa_vs(const Geom g, const T* __restrict__ src, TO* __restrict__ dst, const AaVsCfg cfg, const NormOut no,
         unsigned int* fault)
 {
@@ -80,63 +81,71 @@ bool aa_wide_config(const Geom& g, int method, AaWideCfg& c)
     return false;
 }
 
-// The vertical-first form: output rows no more than source rows; NA = 4, 6
-// or 8 register slots, the fewest with every slot's next row starting at or
-// below the previous row's last tap; the widest power-of-two tile (up to 256
-// columns) whose footprint fits 4 elements per thread; copy-ring chunks of 8
-// rows (4, 2 for wide FP32 rows); bands of the tallest TH (64 .. 8 rows)
-// that still gives at least 4 blocks per SM in all and fits ~75 KB of
-// shared memory, else the shortest that fits the per-block limit.
+// Upper bound of the source samples that the taps of k consecutive outputs
+// span on axis n -> m: floor(x + d) - floor(x) <= ceil(d).
+static int aa_span_bound(int k, int n, int m, int method)
+{
+    const int64_t d = (int64_t)(k - 1) * n + 2 * (int64_t)(method == M_BILINEAR ? 1 : 2) * std::max(n, m);
+    return (int)std::min<int64_t>(n, (d + m - 1) / m);
+}
+
+// The vertical-first form: output rows no more than source rows, and 8 output
+// columns' footprint at most 1024 elements. Tiles: the fewest of equal width
+// whose footprints fit a block (a partly filled tile would cost as much as a
+// full one), with as few warps as hold them. Bands: 3 to 16 blocks per SM,
+// the count with the least rows per SM, counting the rows a band re-reads
+// above it and its start-up (tables, first copies: ~20 rows); with fewer than
+// three blocks on an SM its latencies show.
 bool aa_vs_config(const Geom& g, int method, int dtype, AaVsCfg& c)
 {
     if (method != M_BILINEAR && method != M_BICUBIC) return false;
     if (g.C < 1 || g.C > 4 || g.Ho > g.H) return false;
-    const int es = (int)dtype_size(dtype);
+    const int es = (int)dtype_size(dtype), E = vs_elems(es), cap = kVsNT * E;
     c.method = method;
-    std::vector<int> lo(g.Ho), hi(g.Ho);
-    for (int i = 0; i < g.Ho; ++i) aa_range(i, g.H, g.Ho, method, lo[i], hi[i]);
-    c.NA = 0;
-    for (int na : {4, 6, 8}) {
-        bool ok = true;
-        for (int i = 0; i + na < g.Ho && ok; ++i) ok = lo[i + na] >= hi[i];
-        if (ok) {
-            c.NA = na;
-            break;
-        }
-    }
-    if (!c.NA) return false;
-    c.TW = 0;
-    int span = 0;
-    for (int tw = 256; tw >= 8 && !c.TW; tw /= 2) {
+    c.NA = method == M_BILINEAR ? 2 : 4;
+    int s8 = aa_span_bound(std::min(8, g.Wo), g.W, g.Wo, method);
+    if (s8 * g.C > 1024) {
         int kx = 0;
-        aa_axis_bounds(g.W, g.Wo, method, tw, kx, span);
-        if ((int64_t)span * g.C <= (int64_t)kVsNT * kVsE) {
-            c.TW = tw;
-            c.KX = kx;
-        }
+        aa_axis_bounds(g.W, g.Wo, method, 8, kx, s8);
+        if (s8 * g.C > 1024) return false;
     }
-    if (!c.TW) return false;
-    c.ve = (span * g.C + 3) & ~3;
-    c.raw_row = ((span * g.C * es + 15) / 16 + 2) * 16;   // a spare block past the copied ones
-    c.chunk = 8;
-    while (c.chunk > 2 && (size_t)3 * c.chunk * c.raw_row > 40 * 1024) c.chunk /= 2;
-    const int64_t tiles_x = (g.Wo + c.TW - 1) / c.TW;
+    c.KX = aa_span_bound(1, g.W, g.Wo, method);
+    int tw = 1;
+    while (tw < std::min(g.Wo, 1024) && aa_span_bound(tw + 1, g.W, g.Wo, method) * g.C <= cap) ++tw;
+    const int tiles = (g.Wo + tw - 1) / tw;
+    c.TW = (g.Wo + tiles - 1) / tiles;
+    const int span = aa_span_bound(c.TW, g.W, g.Wo, method);
+    if (span * g.C > cap) return false;
+    c.ve = (span * g.C + E - 1) / E * E;
+    c.nt = std::min(kVsNT, (c.ve / E + 31) / 32 * 32);
+    c.raw_row = std::max((span * g.C * es + 15) / 16 + 2, (15 + span * g.C * es + 4 * vs_words(es) + 15) / 16) * 16;
+    c.chunk = es == 4 ? 2 : 4;
+    const int S = c.raw_row + (int)((g.src_pitch * es) & 15);
+    const double f = (double)g.H / g.Ho, reach = 2.0 * (method == M_BILINEAR ? 1 : 2) * f + 20.0;
+    const int64_t cols = (int64_t)((g.Wo + c.TW - 1) / c.TW) * g.planes;
+    const double sms = num_sms();
     bool any = false;
+    double best = 0.0;
     AaVsCfg fit = c;
-    for (int th = 64; th >= 8; th /= 2) {
-        int ky = 0, nr = 0;
-        aa_axis_bounds(g.H, g.Ho, method, th, ky, nr);
+    for (int k = 3; k <= 16; ++k) {   // blocks per SM
+        const int64_t bands = std::max<int64_t>(1, k * (int64_t)sms / cols);
         AaVsCfg t = c;
-        t.TH = th;
-        t.nr = nr;
-        t.smem = (size_t)3 * t.chunk * t.raw_row +
-                 sizeof(float) * (kVsNB * (size_t)t.ve + (size_t)t.TW * t.KX + (size_t)nr * t.NA) +
-                 sizeof(int) * (2 * (size_t)t.TW + 2 * (size_t)nr);
+        t.TH = (int)std::max<int64_t>(1, (g.Ho + bands - 1) / bands);
+        for (;; t.TH = (t.TH + 1) / 2) {
+            t.nr = aa_span_bound(t.TH, g.H, g.Ho, method);
+            t.smem = 3 * (size_t)vs_rows_bytes(t.chunk, S) + sizeof(float2) * (2 * (size_t)t.ve + (size_t)t.nr * t.NA) +
+                     sizeof(float) * (size_t)t.TW * t.KX + sizeof(int) * (2 * (size_t)t.TW + t.TH);
+            if (t.smem <= max_smem_per_block() || t.TH == 1) break;
+        }
         if (t.smem > max_smem_per_block()) continue;
-        fit = t;
-        any = true;
-        const int64_t blocks = tiles_x * ((g.Ho + th - 1) / th) * g.planes;
-        if (t.smem <= 75 * 1024 && blocks >= 4LL * num_sms()) break;
+        const double per_sm = std::ceil(cols * ((g.Ho + t.TH - 1) / t.TH) / sms);
+        const double resident = std::max(1.0, std::floor(224.0 * 1024 / (t.smem + 1024)));
+        const double cost = per_sm * (t.TH * f + reach) * std::max(1.0, 3.0 / std::min(resident, per_sm));
+        if (!any || cost < best) {
+            fit = t;
+            best = cost;
+            any = true;
+        }
     }
     if (any) c = fit;
     return any;
@@ -152,20 +161,19 @@ static void* aa_vs_func(int C)
 template <typename T, typename TO, bool NORM>
 static void* aa_vs_func_na(int NA, int C)
 {
-    return NA == 4 ? aa_vs_func<T, TO, NORM, 4>(C) : NA == 6 ? aa_vs_func<T, TO, NORM, 6>(C)
-                   : aa_vs_func<T, TO, NORM, 8>(C);
+    return NA == 2 ? aa_vs_func<T, TO, NORM, 2>(C) : aa_vs_func<T, TO, NORM, 4>(C);
 }
 
 static cudaError_t launch_aa_vs_common(const Geom& g, void* func, const void* src, void* dst, const AaVsCfg& c,
                                        const NormOut& no, cudaStream_t st)
 {
-    cudaError_t e = prepare_kernel(func, c.smem, kVsNT, nullptr);
+    cudaError_t e = prepare_kernel(func, c.smem, c.nt, nullptr);
     if (e != cudaSuccess) return e;
     dim3 grid((unsigned)((g.Wo + c.TW - 1) / c.TW), (unsigned)((g.Ho + c.TH - 1) / c.TH), (unsigned)g.planes);
     unsigned int* fw = fault_word();
     void* args[] = {const_cast<Geom*>(&g), const_cast<void**>(&src), &dst, const_cast<AaVsCfg*>(&c),
                     const_cast<NormOut*>(&no), &fw};
-    e = cudaLaunchKernel(func, grid, dim3(kVsNT), args, c.smem, st);
+    e = cudaLaunchKernel(func, grid, dim3(c.nt), args, c.smem, st);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 

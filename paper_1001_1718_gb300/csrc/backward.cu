@@ -876,8 +876,7 @@ static AxisRanges aa_ranges(int n, int m, int method)
 // chunks of 8 staged rows, else 4 (K = 4: large FP32 footprints), else 16.
 static bool aa_window_setup(const Geom& gf, int method, int dtype, int& K, WinCfg& c)
 {
-    const int k = antialias_taps(gf, method);
-    K = k <= 4 ? 4 : k <= 8 ? 8 : 0;
+    K = antialias_capacity(gf, method);
     if (!K) return false;
     for (int ch : {8, 4, 16}) {
         if (ch % K) continue;

@@ -314,8 +314,7 @@ static rs_status prepare_image_aa(const rs_image_desc& x, const Geom& g, int dty
 {
     if (x.method != RS_BILINEAR && x.method != RS_BICUBIC) return RS_ERR_INVALID_ARG;
     im.aa = x.method == RS_BILINEAR ? M_BILINEAR : M_BICUBIC;
-    const int k = antialias_taps(g, im.aa);
-    const int K = k <= 4 ? 4 : k <= 8 ? 8 : 0;
+    const int K = antialias_capacity(g, im.aa);
     // chunks of 8 staged rows, else 4 (K = 4), else 16, within the
     // small-footprint budget; else the same within ~100 KB
     const int chunks[3] = {sh.chunk ? sh.chunk : 8, sh.chunk ? 0 : 4, sh.chunk ? 0 : 16};

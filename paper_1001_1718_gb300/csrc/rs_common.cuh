@@ -24,8 +24,8 @@ namespace rs {
 // first, the quotient is estimated in FP32 and then corrected in exact
 // integer arithmetic, so i0 is exact and t takes a single rounding (the
 // remainder and den are exact FP32 integers). All of it in 32 bits: j, step,
-// first and den are below 2^17 and exact in FP32, the estimate's relative
-// error is below 2^-21 and the quotient below 2^16 in magnitude, so it is
+// first and den are below 2^19 and exact in FP32, the estimate's relative
+// error is below 2^-21 and the quotient below 2^18 in magnitude, so it is
 // off by less than 1; the remainder before the correction lies in (-den, 2 den),
 // so its low 32 bits (wrapping products) hold it. (In 64-bit integers a map
 // cost ~100 instructions, a tenth of the uint8 window kernel's at bands of
@@ -192,7 +192,10 @@ __device__ __forceinline__ void report_fault(unsigned int* fault, unsigned int c
 // u = ((2i+1) m - (2j+1) n) / (2F) kernel units. (Where that bound is an
 // exact integer an FP64 evaluation may add or drop the boundary tap; its
 // weight K(+-R) is zero.) The weights are evaluated in FP32.
-__host__ __device__ inline int64_t floor_div_i64(int64_t a, int64_t b)   // b > 0
+// (2j + 1) n - 2 R F + m = j 2n + (n + m - 2 R F): floor_ratio's form, whose
+// bounds hold (|n + m - 2 R F| < 2^19 is exact in FP32 and the quotients
+// are below 2^18 in magnitude); the difference in u fits in 32 bits.
+inline int64_t floor_div_i64(int64_t a, int64_t b)   // b > 0
 {
     const int64_t q = a / b;
     return (a % b != 0 && a < 0) ? q - 1 : q;
@@ -200,21 +203,29 @@ __host__ __device__ inline int64_t floor_div_i64(int64_t a, int64_t b)   // b > 
 
 __host__ __device__ inline void aa_range(int j, int n, int m, int method, int& lo, int& hi)
 {
-    const int64_t R = method == M_BILINEAR ? 1 : 2;
-    const int64_t F = n > m ? n : m;
+    const int R = method == M_BILINEAR ? 1 : 2;
+    const int F = n > m ? n : m;
+#ifdef __CUDA_ARCH__
+    int rem;
+    const int l = floor_ratio(j, 2 * n, n + m - 2 * R * F, 2 * m, rem);
+    const int h = floor_ratio(j, 2 * n, n + m + 2 * R * F, 2 * m, rem);
+#else
     const int64_t a = (int64_t)(2 * j + 1) * n + m;
-    const int64_t l = floor_div_i64(a - 2 * R * F, 2 * (int64_t)m);
-    const int64_t h = floor_div_i64(a + 2 * R * F, 2 * (int64_t)m);
-    lo = (int)(l < 0 ? 0 : l);
-    hi = (int)(h > n ? n : h);   // exclusive
+    const int l = (int)floor_div_i64(a - 2 * (int64_t)R * F, 2 * (int64_t)m);
+    const int h = (int)floor_div_i64(a + 2 * (int64_t)R * F, 2 * (int64_t)m);
+#endif
+    lo = l < 0 ? 0 : l;
+    hi = h > n ? n : h;   // exclusive
 }
 
-// Unnormalised antialias weight of source index i for the output whose
-// centre is cj / (2 n) (cj = (2 j + 1) n): the kernel at the stretched
-// distance u = |(2 i + 1) m - cj| / (2 max(n, m)).
-__device__ __forceinline__ float aa_kernel(int i, int m, int64_t cj, float inv2F, int method, float a)
+// Unnormalised antialias weight of source index i for output j (centre
+// (2 j + 1) n / (2 m)): the kernel at the stretched distance
+// u = |(2 i + 1) m - (2 j + 1) n| / (2 max(n, m)).
+__device__ __forceinline__ float aa_kernel(int i, int j, int n, int m, float inv2F, int method, float a)
 {
-    const float u = fabsf((float)((int64_t)(2 * i + 1) * m - cj) * inv2F);
+    // |difference| < 2^19 at a tap: its low 32 bits are it
+    const int diff = (int)((uint32_t)(2 * i + 1) * (uint32_t)m - (uint32_t)(2 * j + 1) * (uint32_t)n);
+    const float u = fabsf((float)diff * inv2F);
     if (method == M_BILINEAR) return fmaxf(0.0f, 1.0f - u);
     if (u <= 1.0f) return ((a + 2.0f) * u - (a + 3.0f)) * u * u + 1.0f;
     if (u < 2.0f) return ((a * u - 5.0f * a) * u + 8.0f * a) * u - 4.0f * a;
@@ -233,11 +244,10 @@ __device__ __forceinline__ void aa_taps(int j, int n, int m, int method, float a
         cnt = K;
     }
     const float inv2F = 1.0f / (2.0f * (float)max(n, m));
-    const int64_t cj = (int64_t)(2 * j + 1) * n;
     float tot = 0.0f;
     #pragma unroll
     for (int k = 0; k < K; ++k) {
-        const float v = k < cnt ? aa_kernel(lo + k, m, cj, inv2F, method, a) : 0.0f;
+        const float v = k < cnt ? aa_kernel(lo + k, j, n, m, inv2F, method, a) : 0.0f;
         w[k] = v;
         tot += v;
     }
@@ -253,10 +263,9 @@ __device__ __forceinline__ float aa_weight(int j, int i, int n, int m, int metho
     int lo, hi;
     aa_range(j, n, m, method, lo, hi);
     const float inv2F = 1.0f / (2.0f * (float)max(n, m));
-    const int64_t cj = (int64_t)(2 * j + 1) * n;
     float tot = 0.0f, wi = 0.0f;
     for (int t = lo; t < hi; ++t) {
-        const float v = aa_kernel(t, m, cj, inv2F, method, a);
+        const float v = aa_kernel(t, j, n, m, inv2F, method, a);
         tot += v;
         if (t == i) wi = v;
     }
@@ -276,10 +285,9 @@ __device__ __forceinline__ int aa_taps_n(int j, int n, int m, int method, float 
         cnt = K;
     }
     const float inv2F = 1.0f / (2.0f * (float)max(n, m));
-    const int64_t cj = (int64_t)(2 * j + 1) * n;
     float tot = 0.0f;
     for (int k = 0; k < cnt; ++k) {
-        const float v = aa_kernel(lo + k, m, cj, inv2F, method, a);
+        const float v = aa_kernel(lo + k, j, n, m, inv2F, method, a);
         w[k] = v;
         tot += v;
     }

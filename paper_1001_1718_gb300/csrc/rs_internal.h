@@ -125,13 +125,13 @@ struct AaWideCfg {
 };
 
 // Antialiased vertical downscales, vertical pass first (aa_vs.cuh): tiles
-// of TW output columns x TH rows; KX = the most x taps of an output; NA =
-// register slots of the streamed rows (4, 6 or 8); ve = floats of a finished
-// row buffer (the widest tile footprint times the channels, rounded up to 4;
-// at most 4 per thread); nr = the most source rows of a band of TH output
-// rows; chunk = rows per copy-ring slot; raw_row = bytes per raw ring row.
+// of TW output columns x TH rows, nt threads; KX = the most x taps of an
+// output; NA = sets of vertical sums (2 bilinear, 4 bicubic); ve = elements
+// of a finished row (the widest tile footprint times the channels, rounded up
+// to a thread's); nr = the most source rows of a band of TH output rows;
+// chunk = rows per copy-ring slot; raw_row = bytes per raw ring row.
 struct AaVsCfg {
-    int KX, TW, TH, NA, ve, nr, chunk, raw_row, method;
+    int KX, TW, TH, NA, ve, nr, chunk, raw_row, method, nt;
     size_t smem;
 };
 
@@ -196,9 +196,10 @@ cudaError_t launch_win_raw_norm(const Geom& g, int method, const void* src, void
 cudaError_t launch_win(const Geom& g, int method, int dtype, const void* src, void* dst, WinCfg c, cudaStream_t st);
 // Antialiased resampling (RS_FLAG_ANTIALIAS) on the general window form:
 // the most taps any output has on either axis (antialias_taps), the tap
-// capacity K (4 or 8; 0: too many), configuration and launch (out_dtype /
+// capacity K (antialias_capacity: 4 or 8; 0: too many), configuration and launch (out_dtype /
 // no: the fused pre-process's normalised planar output when norm is set).
 int antialias_taps(const Geom& g, int method);
+int antialias_capacity(const Geom& g, int method);
 bool win_config_aa(const Geom& g, int method, int dtype, int K, WinCfg& c);
 cudaError_t launch_win_aa(const Geom& g, int method, int dtype, const void* src, void* dst, int K, WinCfg c,
                           cudaStream_t st);

@@ -165,6 +165,21 @@ int antialias_taps(const Geom& g, int method)
     return std::max(aa_axis_taps(g.H, g.Ho, method), aa_axis_taps(g.W, g.Wo, method));
 }
 
+// The window forms' tap capacity: 4, 8, or 0 (more taps). The middle outputs
+// decide most problems: their taps are the most, or one less than the bound
+// ceil(2 R F / m); the rest count every output's.
+int antialias_capacity(const Geom& g, int method)
+{
+    auto middle = [&](int n, int m) {
+        int lo, hi;
+        aa_range(m / 2, n, m, method, lo, hi);
+        return hi - lo;
+    };
+    if (std::max(middle(g.H, g.Ho), middle(g.W, g.Wo)) > 8) return 0;
+    const int k = antialias_taps(g, method);
+    return k <= 4 ? 4 : k <= 8 ? 8 : 0;
+}
+
 bool win_config_aa(const Geom& g, int method, int dtype, int K, WinCfg& c)
 {
     if ((method != M_BILINEAR && method != M_BICUBIC) || (K != 4 && K != 8)) return false;
