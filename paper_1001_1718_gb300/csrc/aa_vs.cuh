@@ -9,7 +9,9 @@
 // once, top to bottom. Rows are copied with 16-byte cp.async (one warp per
 // row, rows lying the source pitch mod 16 apart so that every row keeps its
 // address mod 16) into a three-slot ring of R-row chunks, two chunks ahead.
-// Thread t owns footprint elements E t .. E t + E - 1: it reads them as words,
+// Thread t owns footprint elements E t .. E t + E - 1: it reads them as words
+// (AL: where the rows lie a whole number of E elements apart, in one aligned
+// load, the ownership starting up to E - 1 elements before the footprint),
 // widens them and adds the row, weighted, into NA sets of sums, one for every
 // output row whose taps can include the row at once (2 bilinear, 4 bicubic:
 // the stretched kernel is NA output steps long, and output row i + NA starts
@@ -18,13 +20,16 @@
 // unrolled four times, so the sets are registers with fixed roles: row i is
 // complete where its taps end. Four complete rows go to shared memory as two
 // interleaved pairs, and between two barriers the block blends them with the
-// x taps, two rows per packed FMA, and stores the outputs. Sums run over the
-// taps in ascending order, y first, then x.
+// x taps (a thread per output column, two rows per packed FMA) and stores the
+// outputs. Sums run over the taps in ascending order, y first, then x.
 //
-// What bounds it: instruction issue. The form it replaces (4 elements per
-// thread read byte by byte, sums in slots selected at run time, tiles of a
-// power-of-two width) issued 134 M warp instructions for 16 RGB 1080p frames
-// to 455 x 256 and took 177 us; see launch_aa_vs for this one's.
+// What bounds it: instruction issue at 16 warps per SM (16 RGB 1080p frames to
+// 455 x 256, bilinear: 34 M warp instructions, about half the issue slots; 36
+// per source row and warp, a quarter of all in the blend, a tenth in a
+// block's start-up). The form it replaces (4 elements per thread read byte by
+// byte, sums in slots selected at run time, tiles of a power-of-two width)
+// issued 134 M. Measured: 177 -> 62 us; with the words read by funnel shifts
+// at every pitch 70; five blocks of 96 registers per SM 67.
 #pragma once
 
 #include <type_traits>
@@ -42,7 +47,7 @@ constexpr __host__ __device__ int vs_words(int es) { return vs_elems(es) * es / 
 // Shared memory of n rows lying S bytes apart from any 16-byte phase on.
 constexpr __host__ __device__ int vs_rows_bytes(int n, int S) { return (n * S + 31) & ~15; }
 
-template <int C, typename T, typename TO, bool NORM, int NA>
+template <int C, typename T, typename TO, bool NORM, int NA, bool AL>
 __device__ __forceinline__ void aa_vs_body(const Geom& g, const T* __restrict__ s, TO* __restrict__ d,
                                            const AaVsCfg& cfg, int bx, int by, float* sm, unsigned int* fault,
                                            const NormOut& no)
@@ -59,7 +64,10 @@ __device__ __forceinline__ void aa_vs_body(const Geom& g, const T* __restrict__ 
     aa_range(j0 + nj - 1, g.W, g.Wo, m, t1, px_hi);   // exclusive
     aa_range(i0, g.H, g.Ho, m, r_lo, t0);
     aa_range(i0 + ni - 1, g.H, g.Ho, m, t1, r_hi);
-    const int npx = px_hi - px_lo, nr = r_hi - r_lo, ne = npx * C;
+    // AL: rows lie a thread's bytes apart (or a multiple), so owned elements
+    // can start on their own boundary: sh elements before the footprint
+    const int sh = AL ? (int)(reinterpret_cast<uintptr_t>(s + (int64_t)px_lo * C) % (E * ES)) / ES : 0;
+    const int npx = px_hi - px_lo, nr = r_hi - r_lo, ne = npx * C + sh;
     const int per = (ne * ES + 15) / 16 + 1;   // 16-byte blocks around a row's footprint
     // a thread reads bytes [0, 15 + ne ES + 4 NRD) of a raw row
     if (ne > cfg.ve || ne > NT * E || nr > cfg.nr || (per + 1) * 16 > cfg.raw_row || 15 + ne * ES + 4 * NRD > cfg.raw_row ||
@@ -80,7 +88,7 @@ __device__ __forceinline__ void aa_vs_body(const Geom& g, const T* __restrict__ 
     // ---- copies: rows [y0, y0 + n) of the footprint into the slot at rb ----
     const uintptr_t plane_lo = reinterpret_cast<uintptr_t>(s);
     const uintptr_t plane_hi = reinterpret_cast<uintptr_t>(s + (int64_t)(g.H - 1) * g.src_pitch + (int64_t)g.W * C);
-    const T* const foot = s + (int64_t)r_lo * g.src_pitch + (int64_t)px_lo * C;
+    const T* const foot = s + (int64_t)r_lo * g.src_pitch + (int64_t)px_lo * C - sh;
     auto row_at = [&](unsigned char* rb, int y0) {
         return rb + (int)(reinterpret_cast<uintptr_t>(foot + (int64_t)y0 * g.src_pitch) & 15);
     };
@@ -98,7 +106,7 @@ __device__ __forceinline__ void aa_vs_body(const Geom& g, const T* __restrict__ 
                     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((sdst & ~15u) + 16 * w),
                                  "l"(reinterpret_cast<const void*>(blk + 16 * w)) : "memory");
             } else {   // a block would reach outside the plane: element by element
-                for (int e = lane; e < ne; e += 32) reinterpret_cast<T*>(dst)[e] = rp[e];
+                for (int e = sh + lane; e < ne; e += 32) reinterpret_cast<T*>(dst)[e] = rp[e];
             }
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
@@ -114,7 +122,7 @@ __device__ __forceinline__ void aa_vs_body(const Geom& g, const T* __restrict__ 
             const int j = i - ni;
             int lo = 0;
             CX[j] = aa_taps_n(j0 + j, g.W, g.Wo, m, g.a, cfg.KX, lo, WX + j * cfg.KX, fault);
-            LX[j] = lo - px_lo;
+            LX[j] = (lo - px_lo) * C + sh;
             continue;
         }
         // tile row i: its renormalised y taps into its set's column
@@ -168,8 +176,16 @@ __device__ __forceinline__ void aa_vs_body(const Geom& g, const T* __restrict__ 
     // the row at p into every set
     auto add_row = [&]() {
         uint32_t x[NRD];
-        #pragma unroll
-        for (int k = 0; k < NRD; ++k) x[k] = words[(p >> 2) + k];
+        if constexpr (AL && NW == 2) {
+            const uint2 v = *reinterpret_cast<const uint2*>(reinterpret_cast<const unsigned char*>(sm) + p);
+            x[0] = v.x; x[1] = v.y;
+        } else if constexpr (AL) {
+            const uint4 v = *reinterpret_cast<const uint4*>(reinterpret_cast<const unsigned char*>(sm) + p);
+            x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
+        } else {
+            #pragma unroll
+            for (int k = 0; k < NRD; ++k) x[k] = words[(p >> 2) + k];
+        }
         float2 f[E / 2];
         if constexpr (ES == 4) {
             #pragma unroll
@@ -177,7 +193,7 @@ __device__ __forceinline__ void aa_vs_body(const Geom& g, const T* __restrict__ 
         } else {
             #pragma unroll
             for (int k = 0; k < NW; ++k) {
-                const uint32_t w = __funnelshift_r(x[k], x[k + 1], 8 * p);   // the shift counts mod 32
+                const uint32_t w = AL ? x[k] : __funnelshift_r(x[k], x[k + 1], 8 * p);   // the shift counts mod 32
                 if constexpr (ES == 1) {
                     const float2 M = make_float2(-8388608.0f, -8388608.0f);
                     f[2 * k] = __fadd2_rn(make_float2(__int_as_float(__byte_perm(w, 0x4B000000u, 0x7650)),
@@ -205,8 +221,12 @@ __device__ __forceinline__ void aa_vs_body(const Geom& g, const T* __restrict__ 
         p += S;
         yw += NA;
     };
-    const int njc = nj * C;
     for (int f0 = 0; f0 < ni; f0 += 4) {
+        if (ni - f0 <= 2 && own) {   // no second pair: nothing to blend from it
+            float4* v = reinterpret_cast<float4*>(V + cfg.ve + e0);
+            #pragma unroll
+            for (int k = 0; k < E / 2; ++k) v[k] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        }
         #pragma unroll
         for (int u = 0; u < 4; ++u) {
             if (f0 + u < ni) {   // uniform
@@ -216,8 +236,7 @@ __device__ __forceinline__ void aa_vs_body(const Geom& g, const T* __restrict__ 
                     const int ys = min(yh, y_end);
                     for (; y < ys; ++y) add_row();
                 }
-                constexpr int NAc = NA;
-                float2 (&a)[E / 2] = acc[u % NAc];
+                float2 (&a)[E / 2] = acc[u % NA];
                 if (u & 1) {
                     if (own) {
                         float4* v = reinterpret_cast<float4*>(V + (u >> 1) * (size_t)cfg.ve + e0);
@@ -237,34 +256,39 @@ __device__ __forceinline__ void aa_vs_body(const Geom& g, const T* __restrict__ 
                 for (int k = 0; k < E / 2; ++k) a[k] = make_float2(0.0f, 0.0f);
             }
         }
-        // ---- horizontal pass of rows f0 .. f0 + 3 (those the tile has) ----
+        // ---- horizontal pass of rows f0 .. f0 + 3 (those the tile has), all channels of a column per thread ----
         __syncthreads();   // the row pairs complete
         const int nrow = min(4, ni - f0);
-        for (int e = tid; e < njc; e += NT) {
-            const int j = e / C, c = e - j * C;
-            const float2* v0 = V + LX[j] * C + c;
+        for (int j = tid; j < nj; j += NT) {
+            const float2* v0 = V + LX[j];
             const float2* v1 = v0 + cfg.ve;
             const float* w = WX + j * cfg.KX;
             const int cnt = CX[j];
-            float2 a0 = make_float2(0.0f, 0.0f), a1 = a0;
-            if (nrow > 2) {
-                #pragma unroll 4
-                for (int k = 0; k < cnt; ++k) {
-                    const float2 w2 = make_float2(w[k], w[k]);
-                    a0 = __ffma2_rn(w2, v0[k * C], a0);
-                    a1 = __ffma2_rn(w2, v1[k * C], a1);
-                }
-            } else {
-                #pragma unroll 4
-                for (int k = 0; k < cnt; ++k) a0 = __ffma2_rn(make_float2(w[k], w[k]), v0[k * C], a0);
-            }
-            TO* o = d + (int64_t)(i0 + f0) * g.dst_pitch;
-            if constexpr (NORM) o += c * no.c_stride + j0 + j;
-            else o += (int64_t)(j0 + j) * C + c;
-            const float out[4] = {a0.x, a0.y, a1.x, a1.y};
+            float2 a0[C], a1[C];
             #pragma unroll
-            for (int r = 0; r < 4; ++r)
-                if (r < nrow) Store<TO>::put(o + (int64_t)r * g.dst_pitch, NORM ? fmaf(out[r], no.scale[c], no.bias[c]) : out[r]);
+            for (int c = 0; c < C; ++c) a0[c] = a1[c] = make_float2(0.0f, 0.0f);
+            #pragma unroll 2
+            for (int k = 0; k < cnt; ++k, v0 += C, v1 += C) {
+                const float2 w2 = make_float2(w[k], w[k]);
+                #pragma unroll
+                for (int c = 0; c < C; ++c) {
+                    a0[c] = __ffma2_rn(w2, v0[c], a0[c]);
+                    a1[c] = __ffma2_rn(w2, v1[c], a1[c]);
+                }
+            }
+            TO* o = d + (int64_t)(i0 + f0) * g.dst_pitch + (NORM ? j0 + j : (int64_t)(j0 + j) * C);
+            #pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                if (r < nrow) {
+                    #pragma unroll
+                    for (int c = 0; c < C; ++c) {
+                        const float v = r == 0 ? a0[c].x : r == 1 ? a0[c].y : r == 2 ? a1[c].x : a1[c].y;
+                        if constexpr (NORM) Store<TO>::put(o + c * no.c_stride, fmaf(v, no.scale[c], no.bias[c]));
+                        else Store<TO>::put(o + c, v);
+                    }
+                    o += g.dst_pitch;
+                }
+            }
         }
         __syncthreads();   // the pairs free for the next four rows
     }

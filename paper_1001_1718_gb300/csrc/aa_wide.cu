@@ -11,6 +11,13 @@
 #include "aa_wide.cuh"
 #include "aa_vs.cuh"
 
+// Compiled twice so both kernel sets build in parallel: AA_WIDE_PART 0 (the
+// resize kernels, plus the configurations), 1 (the fused pre-process;
+// aa_wide_norm.cu).
+#ifndef AA_WIDE_PART
+#define AA_WIDE_PART 0
+#endif
+
 namespace rs {
 
 template <int C, typename T, typename TO, bool NORM>
@@ -24,16 +31,18 @@ k_aa_wide(const Geom g, const T* __restrict__ src, TO* __restrict__ dst, const A
                                  sm, fault, no);
 }
 
-template <int C, typename T, typename TO, bool NORM, int NA>
-__global__ void __launch_bounds__(kVsNT, 5)
+template <int C, typename T, typename TO, bool NORM, int NA, bool AL>
+__global__ void __launch_bounds__(kVsNT, 4)
 k_aa_vs(const Geom g, const T* __restrict__ src, TO* __restrict__ dst, const AaVsCfg cfg, const NormOut no,
         unsigned int* fault)
 {
     extern __shared__ __align__(16) float sm[];
     const int plane = blockIdx.z;
-    aa_vs_body<C, T, TO, NORM, NA>(g, src + g.sp.offset(plane), dst + g.dp.offset(plane), cfg, blockIdx.x, blockIdx.y,
+    aa_vs_body<C, T, TO, NORM, NA, AL>(g, src + g.sp.offset(plane), dst + g.dp.offset(plane), cfg, blockIdx.x, blockIdx.y,
                                    sm, fault, no);
 }
+
+#if AA_WIDE_PART == 0
 
 // Largest count and widest span of the antialias taps over the tiles of
 // `tile` consecutive outputs along one axis.
@@ -92,15 +101,18 @@ static int aa_span_bound(int k, int n, int m, int method)
 // The vertical-first form: output rows no more than source rows, and 8 output
 // columns' footprint at most 1024 elements. Tiles: the fewest of equal width
 // whose footprints fit a block (a partly filled tile would cost as much as a
-// full one), with as few warps as hold them. Bands: 3 to 16 blocks per SM,
-// the count with the least rows per SM, counting the rows a band re-reads
-// above it and its start-up (tables, first copies: ~20 rows); with fewer than
-// three blocks on an SM its latencies show.
+// full one), with as few warps as hold them. Bands: blocks for whole waves of
+// the resident ones, the count with the least rows per SM, counting the rows
+// a band re-reads above it and its start-up (tables, first copies: ~20 rows);
+// with fewer than three blocks on an SM its latencies show.
 bool aa_vs_config(const Geom& g, int method, int dtype, AaVsCfg& c)
 {
     if (method != M_BILINEAR && method != M_BICUBIC) return false;
     if (g.C < 1 || g.C > 4 || g.Ho > g.H) return false;
-    const int es = (int)dtype_size(dtype), E = vs_elems(es), cap = kVsNT * E;
+    const int es = (int)dtype_size(dtype), E = vs_elems(es);
+    c.aligned = g.src_pitch % E == 0;
+    const int slack = c.aligned ? E - 1 : 0;   // owned elements before the footprint
+    const int cap = kVsNT * E - slack;
     c.method = method;
     c.NA = method == M_BILINEAR ? 2 : 4;
     int s8 = aa_span_bound(std::min(8, g.Wo), g.W, g.Wo, method);
@@ -116,10 +128,11 @@ bool aa_vs_config(const Geom& g, int method, int dtype, AaVsCfg& c)
     c.TW = (g.Wo + tiles - 1) / tiles;
     const int span = aa_span_bound(c.TW, g.W, g.Wo, method);
     if (span * g.C > cap) return false;
-    c.ve = (span * g.C + E - 1) / E * E;
+    const int elems = span * g.C + slack;
+    c.ve = (elems + E - 1) / E * E;
     c.nt = std::min(kVsNT, (c.ve / E + 31) / 32 * 32);
-    c.raw_row = std::max((span * g.C * es + 15) / 16 + 2, (15 + span * g.C * es + 4 * vs_words(es) + 15) / 16) * 16;
-    c.chunk = es == 4 ? 2 : 4;
+    c.raw_row = std::max((elems * es + 15) / 16 + 2, (15 + elems * es + 4 * vs_words(es) + 15) / 16) * 16;
+    c.chunk = es == 1 ? 8 : 4;
     const int S = c.raw_row + (int)((g.src_pitch * es) & 15);
     const double f = (double)g.H / g.Ho, reach = 2.0 * (method == M_BILINEAR ? 1 : 2) * f + 20.0;
     const int64_t cols = (int64_t)((g.Wo + c.TW - 1) / c.TW) * g.planes;
@@ -127,7 +140,7 @@ bool aa_vs_config(const Geom& g, int method, int dtype, AaVsCfg& c)
     bool any = false;
     double best = 0.0;
     AaVsCfg fit = c;
-    for (int k = 3; k <= 16; ++k) {   // blocks per SM
+    for (int k : {3, 4, 8, 12, 16}) {   // blocks per SM (4 are resident)
         const int64_t bands = std::max<int64_t>(1, k * (int64_t)sms / cols);
         AaVsCfg t = c;
         t.TH = (int)std::max<int64_t>(1, (g.Ho + bands - 1) / bands);
@@ -151,17 +164,20 @@ bool aa_vs_config(const Geom& g, int method, int dtype, AaVsCfg& c)
     return any;
 }
 
-template <typename T, typename TO, bool NORM, int NA>
+#endif
+
+template <typename T, typename TO, bool NORM, int NA, bool AL>
 static void* aa_vs_func(int C)
 {
-    return C == 1 ? (void*)&k_aa_vs<1, T, TO, NORM, NA> : C == 2 ? (void*)&k_aa_vs<2, T, TO, NORM, NA>
-         : C == 3 ? (void*)&k_aa_vs<3, T, TO, NORM, NA> : (void*)&k_aa_vs<4, T, TO, NORM, NA>;
+    return C == 1 ? (void*)&k_aa_vs<1, T, TO, NORM, NA, AL> : C == 2 ? (void*)&k_aa_vs<2, T, TO, NORM, NA, AL>
+         : C == 3 ? (void*)&k_aa_vs<3, T, TO, NORM, NA, AL> : (void*)&k_aa_vs<4, T, TO, NORM, NA, AL>;
 }
 
 template <typename T, typename TO, bool NORM>
-static void* aa_vs_func_na(int NA, int C)
+static void* aa_vs_func_na(const AaVsCfg& c, int C)
 {
-    return NA == 2 ? aa_vs_func<T, TO, NORM, 2>(C) : aa_vs_func<T, TO, NORM, 4>(C);
+    if (c.aligned) return c.NA == 2 ? aa_vs_func<T, TO, NORM, 2, true>(C) : aa_vs_func<T, TO, NORM, 4, true>(C);
+    return c.NA == 2 ? aa_vs_func<T, TO, NORM, 2, false>(C) : aa_vs_func<T, TO, NORM, 4, false>(C);
 }
 
 static cudaError_t launch_aa_vs_common(const Geom& g, void* func, const void* src, void* dst, const AaVsCfg& c,
@@ -177,23 +193,29 @@ static cudaError_t launch_aa_vs_common(const Geom& g, void* func, const void* sr
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
+#if AA_WIDE_PART == 0
+
 cudaError_t launch_aa_vs(const Geom& g, int dtype, const void* src, void* dst, const AaVsCfg& c, cudaStream_t st)
 {
-    void* func = dtype == DT_U8 ? aa_vs_func_na<uint8_t, uint8_t, false>(c.NA, g.C)
-               : dtype == DT_F16 ? aa_vs_func_na<__half, __half, false>(c.NA, g.C)
-               : dtype == DT_BF16 ? aa_vs_func_na<__nv_bfloat16, __nv_bfloat16, false>(c.NA, g.C)
-               : aa_vs_func_na<float, float, false>(c.NA, g.C);
+    void* func = dtype == DT_U8 ? aa_vs_func_na<uint8_t, uint8_t, false>(c, g.C)
+               : dtype == DT_F16 ? aa_vs_func_na<__half, __half, false>(c, g.C)
+               : dtype == DT_BF16 ? aa_vs_func_na<__nv_bfloat16, __nv_bfloat16, false>(c, g.C)
+               : aa_vs_func_na<float, float, false>(c, g.C);
     return launch_aa_vs_common(g, func, src, dst, c, NormOut{}, st);
 }
+
+#else
 
 cudaError_t launch_aa_vs_norm(const Geom& g, int out_dtype, const void* src, void* dst, const AaVsCfg& c,
                               const NormOut& no, cudaStream_t st)
 {
-    void* func = out_dtype == DT_F16 ? aa_vs_func_na<uint8_t, __half, true>(c.NA, g.C)
-               : out_dtype == DT_BF16 ? aa_vs_func_na<uint8_t, __nv_bfloat16, true>(c.NA, g.C)
-               : aa_vs_func_na<uint8_t, float, true>(c.NA, g.C);
+    void* func = out_dtype == DT_F16 ? aa_vs_func_na<uint8_t, __half, true>(c, g.C)
+               : out_dtype == DT_BF16 ? aa_vs_func_na<uint8_t, __nv_bfloat16, true>(c, g.C)
+               : aa_vs_func_na<uint8_t, float, true>(c, g.C);
     return launch_aa_vs_common(g, func, src, dst, c, no, st);
 }
+
+#endif
 
 template <typename T, typename TO, bool NORM>
 static void* aa_wide_func(int C)
@@ -215,6 +237,8 @@ static cudaError_t launch_aa_wide_common(const Geom& g, void* func, const void* 
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
+#if AA_WIDE_PART == 0
+
 cudaError_t launch_aa_wide(const Geom& g, int dtype, const void* src, void* dst, const AaWideCfg& c, cudaStream_t st)
 {
     void* func = dtype == DT_U8 ? aa_wide_func<uint8_t, uint8_t, false>(g.C)
@@ -224,6 +248,8 @@ cudaError_t launch_aa_wide(const Geom& g, int dtype, const void* src, void* dst,
     return launch_aa_wide_common(g, func, src, dst, c, NormOut{}, st);
 }
 
+#else
+
 cudaError_t launch_aa_wide_norm(const Geom& g, int out_dtype, const void* src, void* dst, const AaWideCfg& c,
                                 const NormOut& no, cudaStream_t st)
 {
@@ -232,5 +258,7 @@ cudaError_t launch_aa_wide_norm(const Geom& g, int out_dtype, const void* src, v
                : aa_wide_func<uint8_t, float, true>(g.C);
     return launch_aa_wide_common(g, func, src, dst, c, no, st);
 }
+
+#endif
 
 }  // namespace rs

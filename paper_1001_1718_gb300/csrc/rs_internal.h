@@ -129,9 +129,10 @@ struct AaWideCfg {
 // output; NA = sets of vertical sums (2 bilinear, 4 bicubic); ve = elements
 // of a finished row (the widest tile footprint times the channels, rounded up
 // to a thread's); nr = the most source rows of a band of TH output rows;
-// chunk = rows per copy-ring slot; raw_row = bytes per raw ring row.
+// chunk = rows per copy-ring slot; raw_row = bytes per raw ring row; aligned:
+// the source rows lie a whole number of a thread's elements apart.
 struct AaVsCfg {
-    int KX, TW, TH, NA, ve, nr, chunk, raw_row, method, nt;
+    int KX, TW, TH, NA, ve, nr, chunk, raw_row, method, nt, aligned;
     size_t smem;
 };
 
