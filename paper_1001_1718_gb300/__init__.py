@@ -13,6 +13,7 @@ path.
 from __future__ import annotations
 
 import ctypes
+import struct
 from typing import Sequence
 
 import torch
@@ -106,12 +107,13 @@ def _out_shape(x: torch.Tensor, layout: str, Ho: int, Wo: int) -> tuple:
 
 
 _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_get_device = getattr(torch._C, "_cuda_getDevice", torch.cuda.current_device)
 
 
 def _stream(t: torch.Tensor) -> int:
     """torch's current stream on t's device, as a raw cudaStream_t."""
     if _raw_stream is not None:
-        return _raw_stream(t.device.index)
+        return _raw_stream(t.get_device())
     return torch.cuda.current_stream(t.device).cuda_stream
 
 
@@ -120,8 +122,10 @@ class _on_device:
     the current device), entering torch's device context only when another
     device is current."""
 
+    __slots__ = ("ctx",)
+
     def __init__(self, t: torch.Tensor):
-        self.ctx = None if t.device.index == torch.cuda.current_device() else torch.cuda.device(t.device)
+        self.ctx = None if t.get_device() == _get_device() else torch.cuda.device(t.device)
 
     def __enter__(self):
         if self.ctx is not None:
@@ -132,10 +136,32 @@ class _on_device:
             self.ctx.__exit__(*exc)
 
 
-def _opts(coord, cubic_a, impl, tile, threads, waves=0) -> B.RsOptions:
+# Marshalled arguments of recent calls, by the values they were made from
+# (shapes, strides, dtypes, options; never a tensor's identity or address):
+# building them took about half of a small call. The structures are only read
+# by the library, so calls on several threads may share them.
+_CALLS: dict = {}
+_CALLS_MAX = 512
+
+
+def _remember(key, call) -> None:
+    if len(_CALLS) >= _CALLS_MAX:
+        _CALLS.clear()
+    _CALLS[key] = call
+
+
+def _dense_layout(shape, layout: str) -> B.RsLayout:
+    """rs_layout of a new contiguous tensor of `shape`."""
+    return _layout(torch.empty(shape, dtype=torch.uint8, device="meta"), layout)
+
+
+def _opts(coord, cubic_a, impl, tile, threads, waves=0, antialias=False) -> B.RsOptions:
     tw, th = (tile or (0, 0))
-    return B.options(_code(COORDS, coord, "coord"), float(cubic_a), _code(IMPLS, impl, "impl"),
-                     int(tw), int(th), int(threads), int(waves))
+    o = B.options(_code(COORDS, coord, "coord"), float(cubic_a), _code(IMPLS, impl, "impl"),
+                  int(tw), int(th), int(threads), int(waves))
+    if antialias:
+        o.flags = B.RS_FLAG_ANTIALIAS
+    return o
 
 
 def resize(x: torch.Tensor, size: Sequence[int], method="bilinear", *, layout: str = "hwc",
@@ -150,19 +176,32 @@ def resize(x: torch.Tensor, size: Sequence[int], method="bilinear", *, layout: s
     (see RS_FLAG_ANTIALIAS in include/resample.h)."""
     _require_cuda(x)
     Ho, Wo = int(size[0]), int(size[1])
+    a, threads, waves, antialias = float(cubic_a), int(threads), int(waves), bool(antialias)
+    tw, th = (tile or (0, 0))
+    tile = (int(tw), int(th))
+    key = call = None
     if out is None:
-        out = torch.empty(_out_shape(x, layout, Ho, Wo), dtype=x.dtype, device=x.device)
-    _require_cuda(out)
-    if out.dtype != x.dtype:
-        raise ValueError("out must have the dtype of x")
-    Li, Lo = _layout(x, layout), _layout(out, layout)
-    o = _opts(coord, cubic_a, impl, tile, threads, waves)
-    if antialias:
-        o.flags = B.RS_FLAG_ANTIALIAS
+        key = ("resize", x.shape, x.stride(), x.dtype, Ho, Wo, _code(METHODS, method, "method"), layout,
+               _code(COORDS, coord, "coord"), a, _code(IMPLS, impl, "impl"), tile, threads, waves, antialias)
+        call = _CALLS.get(key)
+    if call is None:
+        shape = _out_shape(x, layout, Ho, Wo)
+        if out is None:
+            Lo = _dense_layout(shape, layout)
+        else:
+            _require_cuda(out)
+            if out.dtype != x.dtype:
+                raise ValueError("out must have the dtype of x")
+            Lo = _layout(out, layout)
+        call = (shape, ctypes.byref(_layout(x, layout)), ctypes.byref(Lo), _dtype(x),
+                _code(METHODS, method, "method"), ctypes.byref(_opts(coord, a, impl, tile, threads, waves, antialias)))
+        if key is not None:
+            _remember(key, call)
+    shape, Li, Lo, dt, m, o = call
+    if out is None:
+        out = torch.empty(shape, dtype=x.dtype, device=x.device)
     with _on_device(x):
-        B.check(lib().rs_resize_ex(x.data_ptr(), ctypes.byref(Li), out.data_ptr(), ctypes.byref(Lo),
-                                   _dtype(x), _code(METHODS, method, "method"), ctypes.byref(o),
-                                   _stream(x)), "rs_resize_ex")
+        B.check(lib().rs_resize_ex(x.data_ptr(), Li, out.data_ptr(), Lo, dt, m, o, _stream(x)), "rs_resize_ex")
     return out
 
 
@@ -186,24 +225,36 @@ def resize_normalize(x: torch.Tensor, size: Sequence[int], method="bilinear", me
     except KeyError:
         raise ValueError(f"unsupported output dtype {dtype}") from None
     Ho, Wo = int(size[0]), int(size[1])
-    batched = x.dim() == 4
-    C = x.shape[-1]
-    shape = (x.shape[0], C, Ho, Wo) if batched else (C, Ho, Wo)
+    a, chunk, antialias = float(cubic_a), int(chunk), bool(antialias)
+    mean, std = tuple(float(v) for v in mean), tuple(float(v) for v in std)
+    key = call = None
+    if out is None:
+        key = ("normalize", x.shape, x.stride(), odt, Ho, Wo, _code(METHODS, method, "method"), mean, std,
+               _code(COORDS, coord, "coord"), a, _code(IMPLS, impl, "impl"), chunk, antialias)
+        call = _CALLS.get(key)
+    if call is None:
+        batched = x.dim() == 4
+        C = x.shape[-1]
+        shape = (x.shape[0], C, Ho, Wo) if batched else (C, Ho, Wo)
+        if out is None:
+            Lo = _dense_layout(shape, "nchw")
+        elif tuple(out.shape) != shape or out.dtype != dtype:
+            raise ValueError(f"out must be {shape} of {dtype}")
+        else:
+            Lo = _layout(out, "nchw")
+        Li = _layout(x, "hwc")
+        if len(mean) != C or len(std) != C:
+            raise ValueError("mean and std need one value per channel")
+        call = (shape, ctypes.byref(Li), ctypes.byref(Lo), _code(METHODS, method, "method"),
+                (ctypes.c_float * C)(*mean), (ctypes.c_float * C)(*std),
+                ctypes.byref(_opts(coord, a, impl, (0, chunk), 0, 0, antialias)))
+        if key is not None:
+            _remember(key, call)
+    shape, Li, Lo, m, cm, cs, o = call
     if out is None:
         out = torch.empty(shape, dtype=dtype, device=x.device)
-    elif tuple(out.shape) != shape or out.dtype != dtype:
-        raise ValueError(f"out must be {shape} of {dtype}")
-    Li, Lo = _layout(x, "hwc"), _layout(out, "nchw")
-    if len(mean) != C or len(std) != C:
-        raise ValueError("mean and std need one value per channel")
-    m = (ctypes.c_float * C)(*[float(v) for v in mean])
-    s = (ctypes.c_float * C)(*[float(v) for v in std])
-    o = _opts(coord, cubic_a, impl, (0, chunk), 0)
-    if antialias:
-        o.flags = B.RS_FLAG_ANTIALIAS
     with _on_device(x):
-        B.check(lib().rs_resize_normalize(x.data_ptr(), ctypes.byref(Li), out.data_ptr(), ctypes.byref(Lo), odt,
-                                          _code(METHODS, method, "method"), m, s, ctypes.byref(o), _stream(x)),
+        B.check(lib().rs_resize_normalize(x.data_ptr(), Li, out.data_ptr(), Lo, odt, m, cm, cs, o, _stream(x)),
                 "rs_resize_normalize")
     return out
 
@@ -213,9 +264,7 @@ def backward_workspace_bytes(grad_out: torch.Tensor, in_hw, method, *, layout="n
     H, W = int(in_hw[0]), int(in_hw[1])
     Lo = _layout(grad_out, layout)
     Li = _layout(torch.empty(_out_shape(grad_out, layout, H, W), dtype=grad_out.dtype, device="meta"), layout)
-    o = _opts(coord, cubic_a, "auto", None, 0)
-    if antialias:
-        o.flags = B.RS_FLAG_ANTIALIAS
+    o = _opts(coord, cubic_a, "auto", None, 0, 0, antialias)
     n = ctypes.c_size_t(0)
     B.check(lib().rs_resize_backward_workspace(ctypes.byref(Lo), ctypes.byref(Li),
                                                _code(METHODS, method, "method"), ctypes.byref(o),
@@ -232,24 +281,31 @@ def resize_backward(grad_out: torch.Tensor, in_hw, method="bilinear", *, layout:
     antialias=True is the adjoint of resize(..., antialias=True)."""
     _require_cuda(grad_out)
     H, W = int(in_hw[0]), int(in_hw[1])
+    a, antialias = float(cubic_a), bool(antialias)
+    key = call = None
     if grad_in is None:
-        grad_in = torch.empty(_out_shape(grad_out, layout, H, W), dtype=grad_out.dtype,
-                              device=grad_out.device)
-    Lo, Li = _layout(grad_out, layout), _layout(grad_in, layout)
-    o = _opts(coord, cubic_a, impl, None, 0)
-    if antialias:
-        o.flags = B.RS_FLAG_ANTIALIAS
-    m = _code(METHODS, method, "method")
-    n = ctypes.c_size_t(0)
-    B.check(lib().rs_resize_backward_workspace(ctypes.byref(Lo), ctypes.byref(Li), m, ctypes.byref(o),
-                                               ctypes.byref(n)), "rs_resize_backward_workspace")
-    if workspace is None or workspace.numel() * workspace.element_size() < n.value:
-        workspace = torch.empty(max(1, n.value), dtype=torch.uint8, device=grad_out.device)
+        key = ("backward", grad_out.shape, grad_out.stride(), grad_out.dtype, H, W, _code(METHODS, method, "method"),
+               layout, _code(COORDS, coord, "coord"), a, _code(IMPLS, impl, "impl"), antialias)
+        call = _CALLS.get(key)
+    if call is None:
+        shape = _out_shape(grad_out, layout, H, W)
+        Lo = ctypes.byref(_layout(grad_out, layout))
+        Li = ctypes.byref(_dense_layout(shape, layout) if grad_in is None else _layout(grad_in, layout))
+        o = ctypes.byref(_opts(coord, a, impl, None, 0, 0, antialias))
+        m = _code(METHODS, method, "method")
+        n = ctypes.c_size_t(0)
+        B.check(lib().rs_resize_backward_workspace(Lo, Li, m, o, ctypes.byref(n)), "rs_resize_backward_workspace")
+        call = (shape, Lo, Li, _dtype(grad_out), m, o, n.value)
+        if key is not None:
+            _remember(key, call)
+    shape, Lo, Li, dt, m, o, nbytes = call
+    if grad_in is None:
+        grad_in = torch.empty(shape, dtype=grad_out.dtype, device=grad_out.device)
+    if workspace is None or workspace.numel() * workspace.element_size() < nbytes:
+        workspace = torch.empty(max(1, nbytes), dtype=torch.uint8, device=grad_out.device)
     with _on_device(grad_out):
-        B.check(lib().rs_resize_backward(grad_out.data_ptr(), ctypes.byref(Lo), grad_in.data_ptr(),
-                                         ctypes.byref(Li), _dtype(grad_out), m, ctypes.byref(o),
-                                         workspace.data_ptr(), n.value, _stream(grad_out)),
-                "rs_resize_backward")
+        B.check(lib().rs_resize_backward(grad_out.data_ptr(), Lo, grad_in.data_ptr(), Li, dt, m, o,
+                                         workspace.data_ptr(), nbytes, _stream(grad_out)), "rs_resize_backward")
     return grad_in
 
 
@@ -272,28 +328,36 @@ class ResizeFn(torch.autograd.Function):
         return gi, None, None, None, None, None
 
 
+_DESC = struct.Struct("=QQ6i2q")   # RsImageDesc
+assert _DESC.size == ctypes.sizeof(B.RsImageDesc)
+
+
 def _descs(srcs, dsts, methods) -> tuple:
     n = len(srcs)
-    arr = (B.RsImageDesc * n)()
-    for k, (s, d) in enumerate(zip(srcs, dsts)):
+    buf = bytearray(n * _DESC.size)
+    codes = [_code(METHODS, methods[k], "method") for k in range(n)]
+    at = 0
+    for s, d, m in zip(srcs, dsts, codes):
         if s.dim() != 3 or d.dim() != 3:
             raise ValueError("batched images are (H, W, C) tensors")
-        if s.stride(2) != 1 or s.stride(1) != s.shape[2] or d.stride(2) != 1 or d.stride(1) != d.shape[2]:
+        (H, W, C), (Ho, Wo, Co) = s.shape, d.shape
+        (sr, sp, sc), (dr, dp, dc) = s.stride(), d.stride()
+        if sc != 1 or sp != C or dc != 1 or dp != Co:
             raise ValueError("batched images need dense pixels (pitched rows are fine)")
-        dd = arr[k]
-        dd.src, dd.dst = s.data_ptr(), d.data_ptr()
-        dd.H, dd.W, dd.C = s.shape
-        dd.Ho, dd.Wo = d.shape[0], d.shape[1]
-        dd.method = _code(METHODS, methods[k], "method")
-        dd.src_pitch, dd.dst_pitch = s.stride(0), d.stride(0)
-    return arr, n
+        _DESC.pack_into(buf, at, s.data_ptr(), d.data_ptr(), H, W, C, Ho, Wo, m, sr, dr)
+        at += _DESC.size
+    return (B.RsImageDesc * n).from_buffer(buf), n
 
 
 def batched_workspace_bytes(srcs, dsts, methods) -> int:
     arr, n = _descs(srcs, dsts, methods)
+    return _batch_bytes(arr, n, _dtype(srcs[0]))
+
+
+def _batch_bytes(arr, n: int, dt: int) -> int:
+    """Workspace bytes of a valid batch of n images (they depend on n alone)."""
     nb = ctypes.c_size_t(0)
-    B.check(lib().rs_resize_batched_workspace(arr, n, _dtype(srcs[0]), ctypes.byref(nb)),
-            "rs_resize_batched_workspace")
+    B.check(lib().rs_resize_batched_workspace(arr, n, dt, ctypes.byref(nb)), "rs_resize_batched_workspace")
     return nb.value
 
 
@@ -309,16 +373,16 @@ def resize_batched(srcs: Sequence[torch.Tensor], sizes, methods, *, coord="asymm
         outs = [torch.empty((int(h), int(w), s.shape[2]), dtype=s.dtype, device=s.device)
                 for s, (h, w) in zip(srcs, sizes)]
     arr, n = _descs(srcs, outs, methods)
-    nb = ctypes.c_size_t(0)
     dt = _dtype(srcs[0])
-    B.check(lib().rs_resize_batched_workspace(arr, n, dt, ctypes.byref(nb)), "rs_resize_batched_workspace")
-    if workspace is None or workspace.numel() * workspace.element_size() < nb.value:
-        workspace = torch.empty(max(1, nb.value), dtype=torch.uint8, device=srcs[0].device)
-    o = _opts(coord, cubic_a, impl, tile, threads)
-    if antialias:
-        o.flags = B.RS_FLAG_ANTIALIAS
+    nbytes = _CALLS.get(("batch", n))   # the call itself checks the descriptors again
+    if nbytes is None:
+        nbytes = _batch_bytes(arr, n, dt)
+        _remember(("batch", n), nbytes)
+    if workspace is None or workspace.numel() * workspace.element_size() < nbytes:
+        workspace = torch.empty(max(1, nbytes), dtype=torch.uint8, device=srcs[0].device)
+    o = _opts(coord, cubic_a, impl, tile, threads, 0, antialias)
     with _on_device(srcs[0]):
-        B.check(lib().rs_resize_batched(arr, n, dt, workspace.data_ptr(), nb.value, ctypes.byref(o),
+        B.check(lib().rs_resize_batched(arr, n, dt, workspace.data_ptr(), nbytes, ctypes.byref(o),
                                         _stream(srcs[0])), "rs_resize_batched")
     return outs
 
@@ -336,9 +400,7 @@ class BatchedPlan:
         dt = _dtype(srcs[0])
         B.check(lib().rs_resize_batched_workspace(arr, n, dt, ctypes.byref(nb)), "rs_resize_batched_workspace")
         self.workspace = torch.empty(max(1, nb.value), dtype=torch.uint8, device=srcs[0].device)
-        o = _opts(coord, cubic_a, impl, tile, threads)
-        if antialias:
-            o.flags = B.RS_FLAG_ANTIALIAS
+        o = _opts(coord, cubic_a, impl, tile, threads, 0, antialias)
         self._plan = ctypes.c_void_p()
         self.device = srcs[0].device
         with torch.cuda.device(self.device):
@@ -353,8 +415,8 @@ class BatchedPlan:
         return n.value
 
     def launch(self, stream: int | None = None) -> None:
-        with torch.cuda.device(self.device):
-            st = torch.cuda.current_stream(self.device).cuda_stream if stream is None else stream
+        with _on_device(self.workspace):
+            st = _stream(self.workspace) if stream is None else stream
             B.check(lib().rs_batched_plan_launch(self._plan, st), "rs_batched_plan_launch")
 
     def close(self) -> None:

@@ -40,6 +40,13 @@ static std::string tune_key(const Geom& g, int method, int dtype)
     return "gpu=" + device_tag() + buf;
 }
 
+bool tune_any()
+{
+    std::lock_guard<std::mutex> lk(g_tune_mu);
+    load_env_once();
+    return !g_tune.empty();
+}
+
 bool tune_lookup(const std::string& key, Tuned& t)
 {
     std::lock_guard<std::mutex> lk(g_tune_mu);
@@ -210,8 +217,10 @@ rs_status choose_kernel(const Geom& g, int method, int dtype, const void* src, c
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
         load_env_once();
-        auto it = g_tune.find(tune_key(g, method, dtype));
-        if (it != g_tune.end() && make_choice(g, method, dtype, src, it->second, k)) return RS_OK;
+        if (!g_tune.empty()) {   // (the key is a string of the problem's class)
+            auto it = g_tune.find(tune_key(g, method, dtype));
+            if (it != g_tune.end() && make_choice(g, method, dtype, src, it->second, k)) return RS_OK;
+        }
     }
     return default_choice(g, method, dtype, src, k) ? RS_OK : RS_ERR_UNSUPPORTED;
 }

@@ -21,6 +21,7 @@
 //    transpose. Every dX element is one fixed-order sum, so the result is
 //    deterministic (no atomics).
 #include <algorithm>
+#include <array>
 #include <climits>
 #include <vector>
 
@@ -29,29 +30,37 @@
 
 namespace rs {
 
-// Exact first tap index on the host (same integer arithmetic as the device).
-static int64_t host_floor_div(int64_t num, int64_t den)
+// Exact first tap indices of an axis on the host (the device's map).
+static std::vector<int> host_first_taps(int n, int m, int method, int coord)
 {
-    int64_t q = num / den;
-    if ((num % den != 0) && (num < 0)) q -= 1;
-    return q;
+    int64_t step, first, den;
+    if (coord == COORD_ASYMMETRIC) { step = n; first = 0; den = m; }
+    else if (coord == COORD_HALF_PIXEL) { step = 2 * (int64_t)n; first = (int64_t)n - m; den = 2 * (int64_t)m; }
+    else if (m > 1) { step = n - 1; first = 0; den = m - 1; }   // align-corners: x = j (n - 1) / (m - 1)
+    else { step = 0; first = 0; den = 1; }
+    if (method == M_NEAREST && coord != COORD_ASYMMETRIC) {   // floor(x + 1/2)
+        step *= 2;
+        first = 2 * first + den;
+        den *= 2;
+    }
+    RatioWalk w(step, first, den);
+    std::vector<int> f(m);
+    for (int j = 0; j < m; ++j) f[j] = (int)w.next() - (method == M_BICUBIC);
+    return f;
 }
 
-static int host_first_tap(int j, int n, int m, int method, int coord)
+// Antialias tap ranges [lo, hi) of an axis (aa_range's integer bounds).
+static void host_aa_ranges(int n, int m, int method, std::vector<int>& lo, std::vector<int>& hi)
 {
-    if (coord == COORD_ALIGN_CORNERS) {   // x = j (n - 1) / (m - 1); 0 for one output
-        const int64_t num = m > 1 ? (int64_t)j * (n - 1) : 0, den = m > 1 ? m - 1 : 1;
-        if (method == M_NEAREST) return (int)host_floor_div(2 * num + den, 2 * den);
-        const int64_t i0 = host_floor_div(num, den);
-        return (int)(method == M_BICUBIC ? i0 - 1 : i0);
+    const int64_t R = method == M_BILINEAR ? 1 : 2, F = std::max(n, m);
+    RatioWalk l(2 * (int64_t)n, (int64_t)n + m - 2 * R * F, 2 * (int64_t)m);
+    RatioWalk h(2 * (int64_t)n, (int64_t)n + m + 2 * R * F, 2 * (int64_t)m);
+    lo.resize(m);
+    hi.resize(m);
+    for (int j = 0; j < m; ++j) {
+        lo[j] = (int)std::max<int64_t>(0, l.next());
+        hi[j] = (int)std::min<int64_t>(n, h.next());
     }
-    if (method == M_NEAREST) {
-        if (coord == COORD_ASYMMETRIC) return (int)host_floor_div((int64_t)j * n, m);
-        return (int)host_floor_div((int64_t)(2 * j + 1) * n, 2 * (int64_t)m);
-    }
-    int64_t i0 = coord == COORD_ASYMMETRIC ? host_floor_div((int64_t)j * n, m)
-                                           : host_floor_div((int64_t)(2 * j + 1) * n - m, 2 * (int64_t)m);
-    return (int)(method == M_BICUBIC ? i0 - 1 : i0);
 }
 
 // Ranges [lo[i], hi[i]] of outputs touching input i (hi < lo when none).
@@ -63,20 +72,21 @@ struct AxisRanges {
 static AxisRanges host_ranges(int n, int m, int method, int coord)
 {
     const int KT = method_taps(method);
-    std::vector<int> first(m);
-    for (int j = 0; j < m; ++j) first[j] = host_first_tap(j, n, m, method, coord);
+    const std::vector<int> first = host_first_taps(n, m, method, coord);
     AxisRanges R;
     R.lo.resize(n);
     R.hi.resize(n);
+    int jl = 0, jh = 0;   // first j with first(j) >= i - KT + 1; first j with first(j) > i
     for (int i = 0; i < n; ++i) {
-        // contributors: first(j) in [lo_i, hi_i] with the border widening
-        const int64_t lo_i = (i == 0) ? INT32_MIN : (int64_t)i - KT + 1;
-        const int64_t hi_i = (i == n - 1) ? INT32_MAX : (int64_t)i;
-        const int jl = (int)(std::lower_bound(first.begin(), first.end(), lo_i) - first.begin());
-        const int jh = (int)(std::upper_bound(first.begin(), first.end(), hi_i) - first.begin()) - 1;
+        // contributors: first(j) in [i - KT + 1, i] with the border widening
+        if (i > 0)
+            while (jl < m && first[jl] < i - KT + 1) ++jl;
+        if (i == n - 1) jh = m;
+        else
+            while (jh < m && first[jh] <= i) ++jh;
         R.lo[i] = jl;
-        R.hi[i] = jh;
-        R.kmax = std::max(R.kmax, jh - jl + 1);
+        R.hi[i] = jh - 1;
+        R.kmax = std::max(R.kmax, jh - jl);
     }
     return R;
 }
@@ -84,17 +94,18 @@ static AxisRanges host_ranges(int n, int m, int method, int coord)
 // Antialias taps (method aa): outputs j with lo(j) <= i < hi(j).
 static AxisRanges host_ranges_aa(int n, int m, int aa)
 {
-    std::vector<int> lo(m), hi(m);
-    for (int j = 0; j < m; ++j) aa_range(j, n, m, aa, lo[j], hi[j]);
+    std::vector<int> lo, hi;
+    host_aa_ranges(n, m, aa, lo, hi);
     AxisRanges R;
     R.lo.resize(n);
     R.hi.resize(n);
+    int jl = 0, jh = 0;   // first j with hi(j) > i; first j with lo(j) > i
     for (int i = 0; i < n; ++i) {
-        const int jl = (int)(std::upper_bound(hi.begin(), hi.end(), i) - hi.begin());
-        const int jh = (int)(std::upper_bound(lo.begin(), lo.end(), i) - lo.begin()) - 1;
+        while (jl < m && hi[jl] <= i) ++jl;
+        while (jh < m && lo[jh] <= i) ++jh;
         R.lo[i] = jl;
-        R.hi[i] = jh;
-        R.kmax = std::max(R.kmax, jh - jl + 1);
+        R.hi[i] = jh - 1;
+        R.kmax = std::max(R.kmax, jh - jl);
     }
     return R;
 }
@@ -705,7 +716,7 @@ struct BwdPlan {
 
 static constexpr size_t kAdjTBudget = (size_t)256 << 20;  // bytes of T per plane group
 
-static BwdPlan plan_tables(const Geom& g, int method, int aa)
+static BwdPlan make_plan(const Geom& g, int method, int aa)
 {
     BwdPlan p;
     p.ry = aa ? host_ranges_aa(g.H, g.Ho, aa) : host_ranges(g.H, g.Ho, method, g.coord);
@@ -724,6 +735,22 @@ static BwdPlan plan_tables(const Geom& g, int method, int aa)
     p.off_t = o; o = align256(o + plane_t * p.group_planes);
     p.ws_bytes = o;
     return p;
+}
+
+// The plan of a geometry: a workspace query and its call, and the calls of a
+// training loop, ask for the same one, so each thread keeps its last.
+static const BwdPlan& plan_tables(const Geom& g, int method, int aa)
+{
+    using Key = std::array<int, 9>;
+    static thread_local Key key{};
+    static thread_local BwdPlan plan;
+    const Key k{g.H, g.W, g.Ho, g.Wo, g.C, g.planes, g.coord, method, aa};
+    if (k != key) {
+        key = Key{};   // (sizes are at least 1: the empty key matches nothing)
+        plan = make_plan(g, method, aa);
+        key = k;
+    }
+    return plan;
 }
 
 // Largest staged footprint over all tiles of `tile` destination indices
@@ -860,14 +887,10 @@ static Geom forward_as_adjoint(const Geom& gf)
 static AxisRanges aa_ranges(int n, int m, int method)
 {
     AxisRanges R;
-    R.lo.resize(m);
-    R.hi.resize(m);
+    host_aa_ranges(n, m, method, R.lo, R.hi);
     for (int j = 0; j < m; ++j) {
-        int lo, hi;
-        aa_range(j, n, m, method, lo, hi);
-        R.lo[j] = lo;
-        R.hi[j] = hi - 1;
-        R.kmax = std::max(R.kmax, hi - lo);
+        R.kmax = std::max(R.kmax, R.hi[j] - R.lo[j]);
+        R.hi[j] -= 1;
     }
     return R;
 }
@@ -962,11 +985,10 @@ static AxisRanges point_ranges(int n, int m, int method, int coord, bool columns
 {
     const int K = method_taps(method);
     AxisRanges R;
-    R.lo.resize(m);
+    R.lo = host_first_taps(n, m, method, coord);
     R.hi.resize(m);
     for (int j = 0; j < m; ++j) {
-        const int f = host_first_tap(j, n, m, method, coord);
-        R.lo[j] = columns ? std::max(f, 0) : f;
+        if (columns) R.lo[j] = std::max(R.lo[j], 0);
         R.hi[j] = R.lo[j] + K - 1;
     }
     R.kmax = K;
@@ -1091,7 +1113,7 @@ rs_status rs_resize_backward(const void* grad_out, const rs_layout* out, void* g
     // make_geom checks pointers, alignment and overlap with src = dX, dst = dY.
     s = make_geom(grad_in, in, grad_out, out, RS_F32, method, o, g);
     if (s != RS_OK) return s;
-    BwdPlan p = plan_tables(g, method, aa);
+    const BwdPlan& p = plan_tables(g, method, aa);
     if (!workspace || workspace_bytes < p.ws_bytes) return RS_ERR_WORKSPACE;
     if (reinterpret_cast<uintptr_t>(workspace) % 256) return RS_ERR_ALIGNMENT;
     {

@@ -529,7 +529,7 @@ static rs_status batch_shape(const rs_image_desc* d, int n, int dtype, const rs_
     if (o.impl != RS_IMPL_AUTO) return RS_ERR_INVALID_ARG;
     sh = BatchShape{false, 0, default_band(d, n)};
     Tuned t;
-    if (tuned && tune_lookup(batch_key(d, n, dtype, o), t)) {
+    if (tuned && tune_any() && tune_lookup(batch_key(d, n, dtype, o), t)) {
         if (t.impl == RS_IMPL_TILED) sh = BatchShape{true, 0, 0};
         else if (t.impl == RS_IMPL_WINDOW && t.tile_w >= 1 && t.tile_w <= kWinMaxBand) sh = BatchShape{false, t.tile_h, t.tile_w};
     }
@@ -770,16 +770,51 @@ static rs_status batch_prepare(const rs_image_desc* d, int n, int dtype, const r
                                items.data(), P.L);
     if (s != RS_OK) return s;
     P.off_start = align256(sizeof(BatchImage) * (size_t)n);
-    P.ws_bytes = P.off_start + sizeof(int64_t) * P.start.size();
+    P.ws_bytes = P.off_start + (sizeof(int64_t) * P.start.size() + 15) / 16 * 16;   // whole 16-byte units
     return RS_OK;
 }
 
-static cudaError_t upload(const BatchPlanHost& P, void* ws, cudaStream_t st)
+// A piece of a work list as a kernel argument: the launch copies it, so the
+// host list may go at once and nothing waits (a pageable copy has to: the
+// request of 24 images kept the GPU idle between calls, 159 us a call).
+struct alignas(16) UploadPiece {
+    static constexpr int kBytes = 16 * 1024;
+    unsigned char b[kBytes];
+};
+
+__global__ void __launch_bounds__(64) k_upload(const __grid_constant__ UploadPiece p, unsigned char* dst, int n)
 {
-    std::vector<char> blob(P.ws_bytes, 0);
+    const int i = 16 * (blockIdx.x * 64 + threadIdx.x);
+    if (i < n) *reinterpret_cast<uint4*>(dst + i) = *reinterpret_cast<const uint4*>(p.b + i);
+}
+
+static constexpr int kUploadPieces = 2;   // lists of up to 32 KB (~200 images); longer ones by a copy
+
+// `wait`: the list is read from other streams too (plans).
+static cudaError_t upload(const BatchPlanHost& P, void* ws, cudaStream_t st, bool wait)
+{
+    const size_t padded = (P.ws_bytes + 15) & ~(size_t)15;
+    std::vector<char> blob(padded, 0);
     std::memcpy(blob.data(), P.imgs.data(), sizeof(BatchImage) * P.imgs.size());
     std::memcpy(blob.data() + P.off_start, P.start.data(), sizeof(int64_t) * P.start.size());
-    cudaError_t e = cudaMemcpyAsync(ws, blob.data(), blob.size(), cudaMemcpyHostToDevice, st);
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(st, &cap);
+    if (e != cudaSuccess) return e;
+    if (cap == cudaStreamCaptureStatusNone && P.ws_bytes % 16 == 0 && padded <= (size_t)kUploadPieces * UploadPiece::kBytes) {
+        for (size_t o = 0; o < padded; o += UploadPiece::kBytes) {
+            UploadPiece piece;
+            int n = (int)std::min<size_t>(UploadPiece::kBytes, padded - o);
+            std::memcpy(piece.b, blob.data() + o, n);
+            unsigned char* dst = static_cast<unsigned char*>(ws) + o;
+            void* args[] = {&piece, &dst, &n};
+            e = cudaLaunchKernel(reinterpret_cast<const void*>(&k_upload), dim3((unsigned)((n / 16 + 63) / 64)), dim3(64),
+                                 args, 0, st);
+            if (e == cudaSuccess) e = cudaGetLastError();
+            if (e != cudaSuccess) return e;
+        }
+        return wait ? cudaStreamSynchronize(st) : cudaSuccess;
+    }
+    e = cudaMemcpyAsync(ws, blob.data(), P.ws_bytes, cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) return e;
     // The host blob dies with this function: wait for the copy to finish.
     return cudaStreamSynchronize(st);
@@ -903,7 +938,7 @@ rs_status rs_resize_batched(const rs_image_desc* d, int n, rs_dtype dtype, void*
     if (s != RS_OK) return s;
     if ((s = check_ws(P, workspace, workspace_bytes)) != RS_OK) return s;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    cudaError_t e = upload(P, workspace, st);
+    cudaError_t e = upload(P, workspace, st, false);
     if (e != cudaSuccess) return cuda_status(e);
     ClassLaunch cls[kClasses];
     int nl = 0;
@@ -924,7 +959,7 @@ rs_status rs_batched_plan_create(const rs_image_desc* d, int n, rs_dtype dtype, 
     if (s != RS_OK) return s;
     if ((s = check_ws(P, workspace, workspace_bytes)) != RS_OK) return s;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    cudaError_t e = upload(P, workspace, st);
+    cudaError_t e = upload(P, workspace, st, true);
     if (e != cudaSuccess) return cuda_status(e);
     ClassLaunch cls[kClasses];
     int nl = 0;
@@ -1019,7 +1054,7 @@ rs_status rs_autotune_batched(const rs_image_desc* d, int n, rs_dtype dtype, voi
             if (i == 0) { result = s; break; }   // the default shape must be valid
             continue;
         }
-        if ((e = upload(P, workspace, st)) != cudaSuccess) break;
+        if ((e = upload(P, workspace, st, true)) != cudaSuccess) break;
         ClassLaunch cls[kClasses];
         int nl = 0;
         if ((e = class_launches(P.L, dtype, oc, workspace, static_cast<char*>(workspace) + P.off_start, cls, nl)) !=

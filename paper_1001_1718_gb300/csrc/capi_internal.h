@@ -57,6 +57,7 @@ cudaError_t launch_reduce(const Geom& g, int method, int dtype, const void* src,
 struct Tuned {
     int impl, tile_w, tile_h, threads, waves;
 };
+bool tune_any();   // anything tuned or loaded
 bool tune_lookup(const std::string& key, Tuned& t);
 void tune_store(const std::string& key, const Tuned& t);
 

@@ -35,6 +35,27 @@ inline int tap_span_bound(int k, int n, int m, int KT, int coord)
     const int64_t num = (int64_t)(k - 1) * an;
     return (int)((num + am - 1) / am) + KT;
 }
+// floor((j step + first) / den) for j = 0, 1, ...: one division at the start,
+// additions from there on (host plans walk whole axes).
+struct RatioWalk {
+    int64_t q, r, qs, rs, den;
+    RatioWalk(int64_t step, int64_t first, int64_t d) : den(d)
+    {
+        q = first / d;
+        r = first % d;
+        if (r < 0) { r += d; --q; }
+        qs = step / d;
+        rs = step % d;
+    }
+    int64_t next()
+    {
+        const int64_t v = q;
+        q += qs;
+        r += rs;
+        if (r >= den) { r -= den; ++q; }
+        return v;
+    }
+};
 enum { DT_U8 = 0, DT_F16 = 1, DT_BF16 = 2, DT_F32 = 3 };
 enum { M_NEAREST = 0, M_BILINEAR = 1, M_BICUBIC = 2 };
 

@@ -151,13 +151,15 @@ bool win_config(const Geom& g, int method, int dtype, WinCfg& c, bool allow_x2)
 // the kernels use).
 static int aa_axis_taps(int n, int m, int method)
 {
-    int k = 0;
+    const int64_t R = method == M_BILINEAR ? 1 : 2, F = std::max(n, m);
+    RatioWalk l(2 * (int64_t)n, (int64_t)n + m - 2 * R * F, 2 * (int64_t)m);
+    RatioWalk h(2 * (int64_t)n, (int64_t)n + m + 2 * R * F, 2 * (int64_t)m);
+    int64_t k = 0;
     for (int j = 0; j < m; ++j) {
-        int lo, hi;
-        aa_range(j, n, m, method, lo, hi);
+        const int64_t lo = std::max<int64_t>(0, l.next()), hi = std::min<int64_t>(n, h.next());
         k = std::max(k, hi - lo);
     }
-    return k;
+    return (int)k;
 }
 
 int antialias_taps(const Geom& g, int method)
