@@ -209,8 +209,8 @@ bool win_config(const Geom& g, int method, int dtype, WinCfg& c, bool allow_x2 =
 // x), its default (c.chunk 0: 8 staged rows at a time, or 4 where 8 leave no
 // room for four blocks per SM) and launches (band_h 0 = from occupancy and
 // waves).
-bool win_raw_config(const Geom& g, int method, int dtype, int nt, int band_cap, WinCfg& c);
-bool win_raw_default(const Geom& g, int method, int dtype, int nt, int band_cap, WinCfg& c);
+bool win_raw_config(const Geom& g, int method, int dtype, int nt, int band_cap, WinCfg& c, bool allow_x2 = true);
+bool win_raw_default(const Geom& g, int method, int dtype, int nt, int band_cap, WinCfg& c, bool allow_x2 = true);
 int win_raw_threads(int Wo, int warp_px);
 cudaError_t launch_win_raw(const Geom& g, int method, const void* src, void* dst, WinCfg c, cudaStream_t st);
 cudaError_t launch_win_raw_norm(const Geom& g, int method, const void* src, void* dst, WinCfg c, const NormOut& no,

@@ -9,8 +9,8 @@
 
 // This file is compiled four times so the kernel sets build in parallel:
 // WIN_PART 0 (uint8 / FP16, general; plus the host configuration and
-// launch), 1 (BF16 / FP32, general), 2 (uint8 / FP16, exact x2) and 3
-// (BF16 / FP32, exact x2); win_p1.cu .. win_p3.cu define the part.
+// launch), 1 (BF16 / FP32, general), 2 (FP16, exact x2) and 3 (BF16 / FP32,
+// exact x2); win_p1.cu .. win_p3.cu define the part.
 #ifndef WIN_PART
 #define WIN_PART 0
 #endif
@@ -75,7 +75,7 @@ void* win_kernel_gen_hi(int method, int dtype, int C)
 #elif WIN_PART == 2
 void* win_kernel_x2_lo(int method, int dtype, int C)
 {
-    return dtype == DT_U8 ? win_func_m<uint8_t>(method, C) : win_func_m<__half>(method, C);
+    return dtype == DT_F16 ? win_func_m<__half>(method, C) : nullptr;   // uint8: win_raw.cu
 }
 #else
 void* win_kernel_x2_hi(int method, int dtype, int C)
@@ -218,6 +218,7 @@ cudaError_t launch_win(const Geom& g, int method, int dtype, const void* src, vo
     if (c.pat) return launch_win_raw(g, method, src, dst, c, st);
     const bool x2 = win_is_x2(g);
     void* func = win_kernel(method, dtype, g.C, x2);
+    if (!func) return cudaErrorInvalidValue;
     int per_sm = 1;
     cudaError_t e = prepare_kernel(func, c.smem, kWinThreads, c.band_h <= 0 ? &per_sm : nullptr);
     if (e != cudaSuccess) return e;

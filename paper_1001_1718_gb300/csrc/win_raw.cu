@@ -19,9 +19,15 @@
 namespace rs {
 
 // 128 threads: four blocks of at most 128 registers a thread per SM (RGB
-// bicubic x1.7, 4096^2: 77.8 us; three blocks of up to 168 registers: 79.9).
+// bicubic x1.7, 4096^2 -> 6964^2: 77.8 us; three blocks of up to 168
+// registers: 79.9); the exact-x2 form five (4096^2 -> 8192^2: 55.4 us; four:
+// 58.2, three: 60.6; the form on FP32 windows it replaces: 77.9).
+// Four channels of whole bicubic runs need a few registers more.
 template <int KT, int C, int PAT, int ST>
-__global__ void __launch_bounds__(kWinThreads, 4)
+constexpr int raw_blocks() { return (PAT == kRawX2 ? 5 : 4) - (KT == 4 && C == 4 && ST == RAW_WORDS); }
+
+template <int KT, int C, int PAT, int ST>
+__global__ void __launch_bounds__(kWinThreads, raw_blocks<KT, C, PAT, ST>())
 k_win_raw(const Geom g, const uint8_t* __restrict__ src, uint8_t* __restrict__ dst, const WinCfg cfg,
           unsigned int* fault)
 {
@@ -32,7 +38,7 @@ k_win_raw(const Geom g, const uint8_t* __restrict__ src, uint8_t* __restrict__ d
 }
 
 template <int KT, int C, int PAT, int ST, typename TO>
-__global__ void __launch_bounds__(kWinThreads, 4)
+__global__ void __launch_bounds__(kWinThreads, raw_blocks<KT, C, PAT, ST>())
 k_win_raw_norm(const Geom g, const uint8_t* __restrict__ src, TO* __restrict__ dst, const WinCfg cfg, const NormOut no,
                unsigned int* fault)
 {
@@ -67,10 +73,11 @@ static void* raw_func_p(int pat, int st, int out_dtype)
 {
 #if WIN_RAW_PART < 2
     (void)out_dtype;
-    return pat == 0 ? raw_func_s<C, 0>(st) : pat == 1 ? raw_func_s<C, 1>(st) : raw_func_s<C, 2>(st);
+    return pat == 0 ? raw_func_s<C, 0>(st) : pat == 1 ? raw_func_s<C, 1>(st) : pat == 2 ? raw_func_s<C, 2>(st)
+                                                                             : raw_func_s<C, kRawX2>(st);
 #else
     return pat == 0 ? norm_func_s<C, 0>(st, out_dtype) : pat == 1 ? norm_func_s<C, 1>(st, out_dtype)
-                                                                  : norm_func_s<C, 2>(st, out_dtype);
+         : pat == 2 ? norm_func_s<C, 2>(st, out_dtype) : norm_func_s<C, kRawX2>(st, out_dtype);
 #endif
 }
 
@@ -114,7 +121,7 @@ int win_raw_threads(int Wo, int warp_px)
     return 32 * best;
 }
 
-bool win_raw_config(const Geom& g, int method, int dtype, int nt, int band_cap, WinCfg& c)
+bool win_raw_config(const Geom& g, int method, int dtype, int nt, int band_cap, WinCfg& c, bool allow_x2)
 {
     c.pat = 0;
     if (dtype != DT_U8 || (method != M_BILINEAR && method != M_BICUBIC) || g.C < 1 || g.C > 4) return false;
@@ -122,10 +129,11 @@ bool win_raw_config(const Geom& g, int method, int dtype, int nt, int band_cap, 
     if (c.chunk < KT || c.chunk % KT || c.chunk > 32 || nt < 32 || nt > kWinThreads || nt % 32) return false;
     int64_t an, am;
     coord_advance(g.W, g.Wo, g.coord, an, am);
-    const int pat = raw_pattern(an, am);
+    const int pat = allow_x2 && win_is_x2(g) ? kRawX2 : raw_pattern(an, am);
     if (pat < 0) return false;
     const int span = tap_span_bound(kRawP * nt, g.W, g.Wo, KT, g.coord) * g.C;
-    const int fw = (pat == 0 ? RawPat<0>::hi(kRawP - 1) : pat == 1 ? RawPat<1>::hi(kRawP - 1) : RawPat<2>::hi(kRawP - 1)) + KT;
+    const int fw = (pat == 0 ? RawPat<0>::hi(kRawP - 1) : pat == 1 ? RawPat<1>::hi(kRawP - 1)
+                    : pat == 2 ? RawPat<2>::hi(kRawP - 1) : RawPat<kRawX2>::hi(kRawP - 1)) + KT;
     const int nr = (fw * g.C + 3) / 4 + 1;   // words a thread reads of a row
     c.nt = nt;
     c.raw_row = std::max((span + 15) / 16 + 2, (15 + span + 4 * nr + 15) / 16) * 16;
@@ -144,14 +152,14 @@ bool win_raw_config(const Geom& g, int method, int dtype, int nt, int band_cap, 
     return true;
 }
 
-bool win_raw_default(const Geom& g, int method, int dtype, int nt, int band_cap, WinCfg& c)
+bool win_raw_default(const Geom& g, int method, int dtype, int nt, int band_cap, WinCfg& c, bool allow_x2)
 {
     const int asked = c.chunk;
     c.pat = 0;
     for (int chunk : {asked ? asked : 8, asked ? 0 : 4}) {
         WinCfg t = c;
         t.chunk = chunk;
-        if (!chunk || !win_raw_config(g, method, dtype, nt, band_cap, t)) continue;
+        if (!chunk || !win_raw_config(g, method, dtype, nt, band_cap, t, allow_x2)) continue;
         c = t;
         if (t.smem * (kWinThreads / nt) <= 56 * 1024) break;
     }
@@ -183,6 +191,7 @@ static cudaError_t launch_raw(const Geom& g, void* func, int strip, const void* 
         const int64_t bands = std::max<int64_t>(1, resident * waves / (strips * g.planes));
         c.band_h = (int)std::min<int64_t>(c.band_cap, std::max<int64_t>(1, (g.Ho + bands - 1) / bands));
     }
+    if (c.pat == kRawX2 + 1 && c.band_h % 2) ++c.band_h;   // bands start on even rows (band_cap is even: Ho is)
     if (c.band_h > c.band_cap) return cudaErrorInvalidValue;
     dim3 grid((unsigned)strips, (unsigned)((g.Ho + c.band_h - 1) / c.band_h), (unsigned)g.planes);
     unsigned int* fw = fault_word();

@@ -43,16 +43,22 @@ namespace rs {
 static constexpr int kRawP = 4;   // output pixels per thread
 
 // Ratio ranges: first-tap offsets [lo(k), hi(k)] of pixel k against pixel 0.
-// PAT 0: r <= 1/2, 1: 1/2 < r <= 1, 2: 1 < r <= 2.
+// PAT 0: r <= 1/2, 1: 1/2 < r <= 1, 2: 1 < r <= 2. PAT 3 is the exact x2 form
+// (the asymmetric map, both axes exactly doubled): pixel 2u and row 2u have
+// t = 0 and are the source samples and window rows themselves, pixel 2u + 1
+// and row 2u + 1 have t = 1/2 and the same weights for every u. A position
+// yields two output rows, there are no row tables, and runs start at even
+// pixels, bands at even rows.
+static constexpr int kRawX2 = 3;
 template <int PAT>
 struct RawPat {
     static __host__ __device__ constexpr int lo(int k)
     {
-        return PAT == 0 ? 0 : PAT == 1 ? (k < 2 ? 0 : 1) : k;
+        return PAT == 0 ? 0 : PAT == 1 ? (k < 2 ? 0 : 1) : PAT == 2 ? k : k >> 1;
     }
     static __host__ __device__ constexpr int hi(int k)
     {
-        return PAT == 0 ? (k == 0 ? 0 : k < 3 ? 1 : 2) : PAT == 1 ? k : 2 * k;
+        return PAT == 0 ? (k == 0 ? 0 : k < 3 ? 1 : 2) : PAT == 1 ? k : PAT == 2 ? 2 * k : k >> 1;
     }
 };
 
@@ -97,6 +103,8 @@ __device__ __forceinline__ void win_body_raw(const Geom& g, const uint8_t* __res
 {
     constexpr bool NORM = sizeof(TO) > 1;
     constexpr bool OVL = raw_overlap(ST, sizeof(TO));
+    constexpr bool X2 = PAT == kRawX2;
+    constexpr int HK = KT / 2 - 1;                 // taps left of a pixel's own sample
     constexpr int P = kRawP;
     constexpr int E = P * C, NV = E / 2;           // elements, register pairs of a row
     constexpr int FW = raw_fw<KT, PAT>();          // footprint pixels
@@ -121,7 +129,8 @@ __device__ __forceinline__ void win_body_raw(const Geom& g, const uint8_t* __res
     const int per = (span + 15) / 16 + 1;         // raw 16-byte blocks per row
     const int in_lo = max(0, -px_lo) * C;         // raw bytes [in_lo, in_hi) are in the image
     const int in_hi = (min(px_hi, g.W - 1) + 1) * C - base;
-    if ((per + 1) * 16 > cfg.raw_row || 15 + span + 4 * NR > cfg.raw_row || nrows > cfg.band_cap) {
+    if ((per + 1) * 16 > cfg.raw_row || 15 + span + 4 * NR > cfg.raw_row || nrows > cfg.band_cap ||
+        (X2 && ((yb | nrows) & 1))) {
         if (tid == 0) report_fault(fault, FAULT_TILE_SRC_SPAN);   // uniform over the block
         return;
     }
@@ -182,12 +191,14 @@ __device__ __forceinline__ void win_body_raw(const Geom& g, const uint8_t* __res
     copy_rows(RING + slot_bytes, rc + R, R);
 
     // ---- row taps ----
+    if constexpr (!X2)
     for (int i = tid; i < nrows; i += NT) {
         float w[KT];
         RF[i] = taps<KT>(yb + i, g.H, g.Ho, g.coord, g.a, w);
         #pragma unroll
         for (int q = 0; q < KT; ++q) RW[i * KT + q] = make_float2(w[q], w[q]);
     }
+    if constexpr (!X2)
     for (int q = tid; q < npos4; q += NT) NC[q] = 0;
 
     // ---- this thread's pixels and their column weights over the ranges ----
@@ -195,8 +206,12 @@ __device__ __forceinline__ void win_body_raw(const Geom& g, const uint8_t* __res
     const int nact = j0 < 0 ? 0 : max(0, min(P, j_hi - j0 + 1));   // pixels of the run inside the image and strip
     constexpr int TW = KT + RP::hi(P - 1) - RP::lo(P - 1);   // widest range
     float wx[P][TW];
+    float whalf[KT];   // X2: the t = 1/2 weights
+    tap_weights<KT>(0.5f, g.a, whalf);
     int toff = 0;   // the footprint's first byte in the raw row, before the row's phase
-    {
+    if constexpr (X2) {
+        if (nact > 0) toff = (j0 / 2 - HK - px_lo) * C;
+    } else {
         int f0 = 0;
         #pragma unroll
         for (int k = 0; k < P; ++k) {
@@ -217,6 +232,7 @@ __device__ __forceinline__ void win_body_raw(const Geom& g, const uint8_t* __res
         }
         if (nact > 0) toff = (f0 - px_lo) * C;
     }
+    if constexpr (!X2) {
     __syncthreads();   // row taps visible, NC cleared
     for (int i0 = tid; i0 < nrows; i0 += NT) {   // rows per position (runs of equal first taps)
         if (i0 == 0 || RF[i0] != RF[i0 - 1]) {
@@ -224,6 +240,7 @@ __device__ __forceinline__ void win_body_raw(const Geom& g, const uint8_t* __res
             while (i0 + len < nrows && RF[i0 + len] == RF[i0]) ++len;
             NC[RF[i0] - b_first] = len;
         }
+    }
     }
     // edge pads of landed rows: bytes outside [in_lo, in_hi) take the edge pixel
     auto padfix = [&](unsigned char* rb, int r0, int n) {
@@ -269,6 +286,15 @@ __device__ __forceinline__ void win_body_raw(const Geom& g, const uint8_t* __res
             float a[P];
             #pragma unroll
             for (int k = 0; k < P; ++k) {
+                if constexpr (X2) {
+                    a[k] = F[RP::lo(k) + HK];
+                    if (k & 1) {
+                        a[k] = whalf[0] * F[RP::lo(k)];
+                        #pragma unroll
+                        for (int t = 1; t < KT; ++t) a[k] = fmaf(whalf[t], F[RP::lo(k) + t], a[k]);
+                    }
+                    continue;
+                }
                 a[k] = wx[k][0] * F[RP::lo(k)];
                 #pragma unroll
                 for (int t = 1; t < KT + RP::hi(k) - RP::lo(k); ++t) a[k] = fmaf(wx[k][t], F[RP::lo(k) + t], a[k]);
@@ -296,9 +322,15 @@ __device__ __forceinline__ void win_body_raw(const Geom& g, const uint8_t* __res
             #pragma unroll
             for (int k = 0; k < P; ++k) {
                 float2 a[CP];
+                if (X2 && !(k & 1)) {
+                    #pragma unroll
+                    for (int c = 0; c < CP; ++c) h[k * CP + c] = F[RP::lo(k) + HK][c];
+                    if constexpr (C == 3) bb[k] = B[RP::lo(k) + HK];
+                    continue;
+                }
                 #pragma unroll
                 for (int t = 0; t < KT + RP::hi(k) - RP::lo(k); ++t) {
-                    const float w = wx[k][t];
+                    const float w = X2 ? whalf[t] : wx[k][t];
                     const float2 w2 = make_float2(w, w);
                     #pragma unroll
                     for (int c = 0; c < CP; ++c)
@@ -387,7 +419,9 @@ __device__ __forceinline__ void win_body_raw(const Geom& g, const uint8_t* __res
     auto blend = [&](const float2* wrow, const int* slot, float2 (&v)[NV]) {
         float2 wr[KT];
         #pragma unroll
-        for (int q = 0; q < KT; q += 2) {
+        for (int q = 0; X2 && q < KT; ++q) wr[q] = make_float2(whalf[q], whalf[q]);
+        #pragma unroll
+        for (int q = 0; !X2 && q < KT; q += 2) {
             const float4 w4 = *reinterpret_cast<const float4*>(wrow + q);
             wr[q] = make_float2(w4.x, w4.y);
             wr[q + 1] = make_float2(w4.z, w4.w);
@@ -435,7 +469,10 @@ __device__ __forceinline__ void win_body_raw(const Geom& g, const uint8_t* __res
         // KT positions at a time (past the band's last: rows that nothing is blended from)
         for (; pos < pend; pos += KT) {
             int nb[KT];
-            if constexpr (KT == 4) {
+            if constexpr (X2) {
+                #pragma unroll
+                for (int u = 0; u < KT; ++u) nb[u] = pos + u < npos;
+            } else if constexpr (KT == 4) {
                 const int4 n4 = *reinterpret_cast<const int4*>(NC + pos);
                 nb[0] = n4.x; nb[1] = n4.y; nb[2] = n4.z; nb[3] = n4.w;
             } else {
@@ -448,6 +485,16 @@ __device__ __forceinline__ void win_body_raw(const Geom& g, const uint8_t* __res
                 int slot[KT];
                 #pragma unroll
                 for (int x = 0; x < KT; ++x) slot[x] = (u + x) % KT;
+                if constexpr (X2) {
+                    if (nb[u]) {   // rows 2u (the window row itself) and 2u + 1
+                        float2 v[NV];
+                        blend(wrow, slot, v);
+                        put(out, win[slot[HK]]);
+                        put(out + g.dst_pitch, v);
+                        out += 2 * g.dst_pitch;
+                    }
+                    continue;
+                }
                 #pragma unroll 1
                 for (int k = nb[u]; k > 0; --k) {
                     float2 v[NV];

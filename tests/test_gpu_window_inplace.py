@@ -55,16 +55,28 @@ def test_ratios(W, Wo, coord):
             check(H, W, 3, Ho, Wo, method, coord, a)
 
 
+# The exact x2 form: runs, warps and strips of doubled widths, one source row
+# to several bands.
+@pytest.mark.parametrize("method", ["bilinear", "bicubic"])
+@pytest.mark.parametrize("W", [1, 2, 3, 31, 62, 63, 64, 124, 247, 248, 249, 256, 257, 500])
+def test_x2(W, method):
+    for k, C in enumerate((1, 2, 3, 4)):
+        for H in (1, 2, 37, 300):
+            check(H, W, C, 2 * H, 2 * W, method, "asymmetric")
+        check(37, W, C, 74, 2 * W, method, "asymmetric", a=-0.75, pad=k + 1, off=k + 3)
+
+
 @pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16, torch.float32])
-@pytest.mark.parametrize("W,Wo", [(100, 257), (300, 512), (455, 455), (700, 455), (1024, 512), (9, 5)])
+@pytest.mark.parametrize("W,Wo", [(100, 257), (300, 512), (455, 455), (700, 455), (1024, 512), (9, 5), (130, 260), (63, 126)])
 def test_normalize(W, Wo, dtype):
     mean, std = (123.675, 116.28, 103.53), (58.395, 57.12, 57.375)
     for C in (1, 3):
         for method, coord in (("bilinear", "half_pixel"), ("bicubic", "asymmetric")):
             _, x = image(W, 41, W, C, 5, 1)
             x2 = torch.stack([x, x.flip(0)])
-            y = rs.resize_normalize(x2, (29, Wo), method, mean[:C], std[:C], dtype=dtype, coord=coord)
-            v = rs.resize(x2.float(), (29, Wo), method, coord=coord, impl="tiled").double().permute(0, 3, 1, 2)
+            Ho = 82 if Wo == 2 * W else 29
+            y = rs.resize_normalize(x2, (Ho, Wo), method, mean[:C], std[:C], dtype=dtype, coord=coord)
+            v = rs.resize(x2.float(), (Ho, Wo), method, coord=coord, impl="tiled").double().permute(0, 3, 1, 2)
             sc = torch.tensor([np.float32(1) / np.float32(s) for s in std[:C]], device="cuda").double().view(1, C, 1, 1)
             bi = torch.tensor([-np.float32(m) / np.float32(s) for m, s in zip(mean, std)][:C], device="cuda").double()
             # one FP32 multiply-add of the FP32 value, then one rounding to the output type
