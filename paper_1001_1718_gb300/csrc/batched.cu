@@ -79,7 +79,16 @@ __device__ __forceinline__ int find_image(const int64_t* __restrict__ start, int
 // drawn while the current one runs. Every block draws until it draws past the
 // end, `total` draws in all (the grid is no larger than `total`), and the
 // last one sets the counter back to 0 for the next launch.
+// The classes of a direct call are launched one behind the other with the next
+// allowed to start while the last items of this one still run (they share
+// nothing but the finished work list): `open` lets it, and `close` holds every
+// block until the class before has ended, so that the last launch's end is the
+// end of all. Both do nothing in a launch without that permission (plans
+// record the classes side by side).
 struct ItemQueue {
+    static __device__ __forceinline__ void open() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+    static __device__ __forceinline__ void close() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
     unsigned long long* next;
     int64_t t, total;
     unsigned long long drawn;   // thread 0
@@ -126,6 +135,7 @@ k_batched_window(const BatchImage* __restrict__ imgs, const int64_t* __restrict_
                  unsigned long long* next, int coord, float a, unsigned int* fault)
 {
     extern __shared__ __align__(16) float sm[];
+    ItemQueue::open();
     for (ItemQueue q(next, total); q.t < total; q.advance()) {
         const int64_t t = q.t;
         const int k = find_image(start, n, t);
@@ -152,6 +162,7 @@ k_batched_window(const BatchImage* __restrict__ imgs, const int64_t* __restrict_
         win_body<KT, C, T, T, false, TM>(g, static_cast<const T*>(im.src), static_cast<T*>(im.dst), wc,
                                          (int)(local % im.tiles_x), (int)(local / im.tiles_x), sm, fault);
     }
+    ItemQueue::close();
 }
 
 // Window items of uint8 sources read in place (kind 3), any ratio range.
@@ -162,6 +173,7 @@ k_batched_raw(const BatchImage* __restrict__ imgs, const int64_t* __restrict__ s
               unsigned long long* next, int coord, float a, unsigned int* fault)
 {
     extern __shared__ __align__(16) float sm[];
+    ItemQueue::open();
     for (ItemQueue q(next, total); q.t < total; q.advance()) {
         const int64_t t = q.t;
         const int k = find_image(start, n, t);
@@ -194,6 +206,7 @@ k_batched_raw(const BatchImage* __restrict__ imgs, const int64_t* __restrict__ s
         else if (im.pat == 1) win_body_raw<KT, C, 0, RAW_ANY>(g, s, d, wc, bx, by, sm, fault);
         else win_body_raw<KT, C, 1, RAW_ANY>(g, s, d, wc, bx, by, sm, fault);
     }
+    ItemQueue::close();
 }
 
 // Many-tap antialias tiles (kind 2) of any channel count.
@@ -203,6 +216,7 @@ k_batched_aa_wide(const BatchImage* __restrict__ imgs, const int64_t* __restrict
                   unsigned long long* next, int coord, float a, unsigned int* fault)
 {
     extern __shared__ __align__(16) float sm[];
+    ItemQueue::open();
     for (ItemQueue q(next, total); q.t < total; q.advance()) {
         const int64_t t = q.t;
         const int k = find_image(start, n, t);
@@ -227,6 +241,7 @@ k_batched_aa_wide(const BatchImage* __restrict__ imgs, const int64_t* __restrict
         default: aa_wide_body<4, T, T, false>(g, s, d, c, bx, by, sm, fault, NormOut{}); break;
         }
     }
+    ItemQueue::close();
 }
 
 template <int KT, typename T>
@@ -250,6 +265,7 @@ k_batched(const BatchImage* __restrict__ imgs, const int64_t* __restrict__ start
           unsigned long long* next, int coord, float a, unsigned int* fault)
 {
     extern __shared__ __align__(16) float sm[];
+    ItemQueue::open();
     for (ItemQueue q(next, total); q.t < total; q.advance()) {
         const int64_t t = q.t;
         const int k = find_image(start, n, t);
@@ -274,6 +290,7 @@ k_batched(const BatchImage* __restrict__ imgs, const int64_t* __restrict__ start
         default: batch_tile_c<4, T>(g, im, cfg, bx, by, sm, fault); break;
         }
     }
+    ItemQueue::close();
 }
 
 // ---------------------------------------------------------------------------
@@ -743,7 +760,17 @@ static cudaError_t launch_classes(ClassLaunch* cls, int nl, cudaStream_t st)
     for (int i = 0; i < nl; ++i) {
         ClassLaunch& c = cls[i];
         void* args[] = {&c.imgs, &c.start, &c.n, &c.total, &c.next, &c.coord, &c.a, &c.fault};
-        cudaError_t e = cudaLaunchKernel(c.func, c.grid, c.block, args, c.smem, st);
+        cudaLaunchAttribute at;
+        at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at.val.programmaticStreamSerializationAllowed = 1;
+        cudaLaunchConfig_t lc{};
+        lc.gridDim = c.grid;
+        lc.blockDim = c.block;
+        lc.dynamicSmemBytes = c.smem;
+        lc.stream = st;
+        lc.attrs = &at;
+        lc.numAttrs = i > 0 ? 1 : 0;   // the first waits for what is before it (its work list)
+        cudaError_t e = cudaLaunchKernelExC(&lc, c.func, args);
         if (e == cudaSuccess) e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
