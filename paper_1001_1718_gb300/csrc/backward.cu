@@ -702,6 +702,219 @@ k_adj_window(const Geom g, const float* __restrict__ dY, float* __restrict__ dX,
 }
 
 // ---------------------------------------------------------------------------
+// Exact-x2 adjoint (one channel, both axes exactly doubled, asymmetric or
+// half-pixel map): input i's outputs are 2 i + c .. 2 i + c + K - 1 for every
+// i, with K = 2 KT, c = -KT (asymmetric) or 1 - KT (half-pixel), and away from
+// the edges the same K weights (two fractions: 0 and 1/2, or 3/4 and 1/4).
+//
+// A block of NT threads owns a strip of 2 NT dX columns and a band of dX
+// rows; thread t owns columns 2 t and 2 t + 1, whose taps of a dY row are at
+// fixed places among 12 consecutive staged floats from 4 t on: three 16-byte
+// shared loads without bank conflicts, no selection. It keeps the last K
+// x-adjointed dY rows in registers; every two rows give one dX row. dY rows
+// are copied with 16-byte cp.async into a three-slot ring of 4-row chunks,
+// two chunks ahead; columns outside the row are zeros, rows outside the image
+// count as zeros. The weights are computed in the kernel (no table pass).
+// Same sums in the same order as the table kernels.
+//
+// What bounds it: HBM (dY once, dX once). k_adj_window on the same problem
+// reads each tap pair at any parity (10 8-byte shared loads and 16 selects
+// per dY row and thread) and was bound by instruction issue; both measured at
+// launch_adj_x2.
+static constexpr int kX2Threads = 256;   // at most
+static constexpr int kX2Chunk = 4;
+
+// First tap of output j.
+template <int KT, bool HALF>
+__device__ __forceinline__ int x2_first(int j) { return (j >> 1) - (KT / 2 - 1) - (HALF && !(j & 1)); }
+
+// Weights of input i (of n) at its K outputs; we / wo: the taps' weights of
+// the even / odd outputs.
+template <int KT, bool HALF>
+__device__ __forceinline__ void x2_weights(int i, int n, const float* we, const float* wo, float* w)
+{
+    constexpr int K = 2 * KT, c = HALF ? 1 - KT : -KT;
+    #pragma unroll
+    for (int t = 0; t < K; ++t) {
+        const int j = 2 * i + c + t, f = x2_first<KT, HALF>(j);
+        float acc = 0.0f;
+        #pragma unroll
+        for (int q = 0; q < KT; ++q)
+            if (clampi(f + q, n) == i) acc += ((c + t) & 1) ? wo[q] : we[q];
+        w[t] = j >= 0 && j < 2 * n ? acc : 0.0f;
+    }
+}
+
+template <int KT, bool HALF>
+__global__ void __launch_bounds__(kX2Threads, 3)
+k_adj_x2(const Geom g, const float* __restrict__ dY, float* __restrict__ dX, int band_h, int row_floats, unsigned int* fault)
+{
+    constexpr int K = 2 * KT, c = HALF ? 1 - KT : -KT, R = kX2Chunk;
+    extern __shared__ __align__(16) float sm[];
+    const int tid = threadIdx.x, NT = blockDim.x;
+    const float* s = dY + g.dp.offset(blockIdx.z);
+    float* d = dX + g.sp.offset(blockIdx.z);
+    const int x0 = blockIdx.x * 2 * NT;
+    const int ncol = min(2 * NT, g.W - x0);
+    const int yb = blockIdx.y * band_h;
+    const int nrows = min(band_h, g.H - yb);
+    // Staged columns [2 x0 - 4, 2 x0 + 2 ncol + 8); in the row: whole 16-byte
+    // units u_lo .. u_hi - 1 of them (x0 and Wo / 2 are even).
+    const int units = (2 * ncol + 12 + 3) / 4;
+    const int u_lo = x0 == 0 ? 1 : 0, u_hi = min(units, (g.Wo - (2 * x0 - 4)) / 4);
+    if (4 * units > row_floats || 4 * (NT + 2) > row_floats || nrows < 1) {   // uniform; the host sizes the rows
+        if (tid == 0) report_fault(fault, FAULT_BWD_SPAN);
+        return;
+    }
+    float* RING = sm;                               // [3][R][row_floats]
+    float* RW = RING + 3 * R * row_floats;          // [band_h][K]
+    const int r_first = 2 * yb + c, r_end = 2 * (yb + nrows - 1) + c + K;   // dY rows, unclamped
+    const uint32_t nu = (uint32_t)max(1, u_hi - u_lo), umul = nu > 1 ? 0xFFFFFFFFu / nu + 1u : 0u;
+    auto issue = [&](int ch) {
+        const int r0 = r_first + ch * R, nn = max(0, min(R, r_end - r0));
+        float* slot = RING + (ch % 3) * R * row_floats;
+        for (int u = tid; u < nn * (int)nu; u += NT) {
+            const int k = nu > 1 ? (int)__umulhi((uint32_t)u, umul) : u;
+            const int w = u_lo + u - k * (int)nu;
+            const float* src = s + (int64_t)clampi(r0 + k, g.Ho) * g.dst_pitch + 2 * x0 - 4 + 4 * w;
+            const unsigned sdst = (unsigned)__cvta_generic_to_shared(slot + k * row_floats + 4 * w);
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sdst), "l"(src) : "memory");
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    issue(0);
+    issue(1);
+    issue(2);
+    // zeros outside the row, in every slot row (the copies leave them)
+    const int pad_hi = row_floats - 4 * u_hi;
+    for (int u = tid; u < 3 * R * (4 * u_lo + pad_hi); u += NT) {
+        const int row = u / (4 * u_lo + pad_hi), q = u - row * (4 * u_lo + pad_hi);
+        RING[row * row_floats + (q < 4 * u_lo ? q : 4 * u_hi + q - 4 * u_lo)] = 0.0f;
+    }
+    float we[KT], wo[KT];
+    tap_weights<KT>(HALF ? 0.75f : 0.0f, g.a, we);
+    tap_weights<KT>(HALF ? 0.25f : 0.5f, g.a, wo);
+    for (int i = tid; i < nrows; i += NT) {
+        float w[K];
+        x2_weights<KT, HALF>(yb + i, g.H, we, wo, w);
+        #pragma unroll
+        for (int t = 0; t < K; ++t) RW[i * K + t] = w[t];
+    }
+    const int i0 = x0 + 2 * tid;
+    const int nact = max(0, min(2, g.W - i0));
+    float wx[2][K];
+    #pragma unroll
+    for (int k = 0; k < 2; ++k)
+        x2_weights<KT, HALF>(i0 + k, g.W, we, wo, wx[k]);
+    asm volatile("cp.async.wait_group 2;" ::: "memory");
+    __syncthreads();   // chunk 0, the pads and the row weights visible
+
+    // x-adjoint of the staged row at Sr (row r of dY)
+    auto hrow = [&](const float* Sr, int r, float2& h) {
+        float f[12];
+        #pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const float4 v = *reinterpret_cast<const float4*>(Sr + 4 * tid + 4 * q);
+            f[4 * q] = v.x; f[4 * q + 1] = v.y; f[4 * q + 2] = v.z; f[4 * q + 3] = v.w;
+        }
+        float a0 = 0.0f, a1 = 0.0f;
+        #pragma unroll
+        for (int t = 0; t < K; ++t) {
+            a0 = fmaf(wx[0][t], f[4 + c + t], a0);
+            a1 = fmaf(wx[1][t], f[6 + c + t], a1);
+        }
+        const bool in = r >= 0 && r < g.Ho;   // uniform
+        h = make_float2(in ? a0 : 0.0f, in ? a1 : 0.0f);
+    };
+    float2 h[K];
+    int r = r_first, ch = 0;
+    const float* Sr = RING;
+    auto next_chunk = [&]() {
+        ++ch;
+        Sr = RING + (ch % 3) * R * row_floats;
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncthreads();   // chunk ch landed; every thread is done with chunk ch - 1
+        issue(ch + 2);
+    };
+    auto take = [&](float2& out) {
+        hrow(Sr, r, out);
+        Sr += row_floats;
+        ++r;
+    };
+    #pragma unroll
+    for (int p = 0; p < K - 2; ++p) {
+        if (p == R) next_chunk();
+        take(h[p]);
+    }
+    float* o = d + (int64_t)yb * g.src_pitch + i0;
+    const bool vec = nact == 2 && ((reinterpret_cast<uintptr_t>(o) | (uintptr_t)(g.src_pitch * 4)) & 7) == 0;
+    const float* rw = RW;
+    for (int i = 0; i < nrows; i += KT) {
+        #pragma unroll
+        for (int u = 0; u < KT; ++u) {   // dX row yb + i + u: rows 2 u .. 2 u + K - 1 of the window
+            if (i + u < nrows) {
+                if (u & 1) next_chunk();   // (K - 2 + 2 u rows taken: whole chunks at odd u)
+                take(h[(2 * u + K - 2) % K]);
+                take(h[(2 * u + K - 1) % K]);
+                float w[K];
+                #pragma unroll
+                for (int t = 0; t < K; t += 4) {
+                    const float4 w4 = *reinterpret_cast<const float4*>(rw + t);
+                    w[t] = w4.x; w[t + 1] = w4.y; w[t + 2] = w4.z; w[t + 3] = w4.w;
+                }
+                float2 v = make_float2(0.0f, 0.0f);
+                #pragma unroll
+                for (int t = 0; t < K; ++t) v = __ffma2_rn(make_float2(w[t], w[t]), h[(2 * u + t) % K], v);
+                if (vec) {
+                    *reinterpret_cast<float2*>(o) = v;
+                } else {
+                    if (nact > 0) o[0] = v.x;
+                    if (nact > 1) o[1] = v.y;
+                }
+                o += g.src_pitch;
+                rw += K;
+            }
+        }
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+}
+
+static bool adj_x2_ok(const Geom& g, int method, int aa, const void* dY)
+{
+    return g.C == 1 && !aa && (method == M_BILINEAR || method == M_BICUBIC) &&
+           (g.coord == COORD_ASYMMETRIC || g.coord == COORD_HALF_PIXEL) && (int64_t)g.Ho == 2 * (int64_t)g.H &&
+           (int64_t)g.Wo == 2 * (int64_t)g.W && g.Wo % 4 == 0 && reinterpret_cast<uintptr_t>(dY) % 16 == 0 &&
+           g.dst_pitch % 4 == 0 && (g.planes == 1 || (g.dp.n_stride % 4 == 0 && g.dp.c_stride % 4 == 0));
+}
+
+static cudaError_t launch_adj_x2(const Geom& g, int method, const float* dY, float* dX, cudaStream_t st)
+{
+    const bool half = g.coord == COORD_HALF_PIXEL;
+    const void* func = method == M_BILINEAR ? (half ? (const void*)&k_adj_x2<2, true> : (const void*)&k_adj_x2<2, false>)
+                                            : (half ? (const void*)&k_adj_x2<4, true> : (const void*)&k_adj_x2<4, false>);
+    const int K = 2 * method_taps(method);
+    // strips of equal width, at most 512 columns
+    const int strips = (g.W + 2 * kX2Threads - 1) / (2 * kX2Threads);
+    int nt = ((g.W + strips - 1) / strips + 1) / 2;
+    nt = (nt + 31) / 32 * 32;
+    const int gx = (g.W + 2 * nt - 1) / (2 * nt);
+    int row_floats = 4 * (nt + 3);   // a strip's units, and every thread's 12 floats
+    const int band_cap = std::min(256, g.H);
+    auto bytes = [&](int band) { return sizeof(float) * (3 * (size_t)kX2Chunk * row_floats + (size_t)band * K); };
+    int per_sm = 1;
+    cudaError_t e = prepare_kernel(func, bytes(band_cap), nt, &per_sm);
+    if (e != cudaSuccess) return e;
+    const int64_t resident = (int64_t)num_sms() * std::max(1, per_sm);
+    const int64_t bands = std::max<int64_t>(1, 2 * resident / ((int64_t)gx * g.planes));   // no partial extra wave
+    int band_h = (int)std::min<int64_t>(band_cap, std::max<int64_t>(1, (g.H + bands - 1) / bands));
+    dim3 grid((unsigned)gx, (unsigned)((g.H + band_h - 1) / band_h), (unsigned)g.planes);
+    unsigned int* fw = fault_word();
+    void* args[] = {const_cast<Geom*>(&g), const_cast<float**>(&dY), &dX, &band_h, &row_floats, &fw};
+    e = cudaLaunchKernel(func, grid, dim3(nt), args, bytes(band_cap), st);
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+// ---------------------------------------------------------------------------
 
 static size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 
@@ -1150,6 +1363,8 @@ rs_status rs_resize_backward(const void* grad_out, const rs_layout* out, void* g
     }
 
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    if (window_ok && adj_x2_ok(g, method, aa, grad_out))
+        return cuda_status(launch_adj_x2(g, method, static_cast<const float*>(grad_out), static_cast<float*>(grad_in), st));
     char* ws = static_cast<char*>(workspace);
     AdjTables tb;
     tb.ylo = reinterpret_cast<int*>(ws + p.off_ylo);
