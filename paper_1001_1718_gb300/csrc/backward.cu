@@ -440,8 +440,8 @@ struct AdjWinCfg {
     size_t smem;
 };
 
-// Threads per block: 256 (strips of 512 dX elements), or 128 (strips of
-// 256) for the computed-tap modes where that pads narrow rows less.
+// Threads per block, at most (strips of 512 dX elements); fewer where the
+// rows are narrow or split evenly into narrower strips (adj_window_config).
 static constexpr int kAwThreads = 256;
 
 // Where the taps come from. TAPS_TABLE: the transposed tables of the
@@ -454,13 +454,13 @@ static constexpr int kAwThreads = 256;
 // consecutive staged columns from max(first tap, 0).
 enum { TAPS_TABLE = 0, TAPS_AA = 1, TAPS_POINT = 2 };
 
-template <int C, int KX, int KY, int TM, int NT = kAwThreads>
-__global__ void __launch_bounds__(NT, 512 / NT)
+template <int C, int KX, int KY, int TM>
+__global__ void __launch_bounds__(kAwThreads, 2)
 k_adj_window(const Geom g, const float* __restrict__ dY, float* __restrict__ dX, const AdjTables tb,
              const AdjWinCfg cfg, unsigned int* fault)
 {
     extern __shared__ __align__(16) float sm[];
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, NT = blockDim.x;
     const int plane = blockIdx.z;
     const float* s = dY + g.dp.offset(plane);   // Ho rows of Wo C, pitch dst_pitch
     float* d = dX + g.sp.offset(plane);         // H rows of W C, pitch src_pitch
@@ -1008,8 +1008,12 @@ static bool adj_window_config(const Geom& g, const BwdPlan& p, const void* dY, A
     if (g.planes > 1 && (g.dp.n_stride % 4 || g.dp.c_stride % 4)) return false;
     c.chunk = std::max(4, KY);
     const int WC = g.W * g.C;
-    // 128-thread blocks where strips of 256 pad the rows less than strips of 512
-    c.nt = narrow && (WC + 255) / 256 * 256 < (WC + 511) / 512 * 512 ? 128 : kAwThreads;
+    // 128-thread blocks where strips of 256 pad the rows less than strips of
+    // 512; then strips of equal width, in whole warps (a 130-wide row in a
+    // 512-wide strip left three quarters of the threads idle)
+    const int most = narrow && (WC + 255) / 256 * 256 < (WC + 511) / 512 * 512 ? 128 : kAwThreads;
+    const int strips = (WC + 2 * most - 1) / (2 * most);
+    c.nt = (((WC + strips - 1) / strips + 1) / 2 + 31) / 32 * 32;
     const int elems = 2 * c.nt;
     int swe = 4;
     for (int e0 = 0; e0 < WC; e0 += elems) {
@@ -1034,33 +1038,25 @@ static bool adj_window_config(const Geom& g, const BwdPlan& p, const void* dY, A
 }
 
 template <int C, int KX, int KY>
-static void* adj_window_func(int tm, int nt)
+static void* adj_window_func(int tm)
 {
-    if (tm == TAPS_AA)
-        return nt == 128 ? reinterpret_cast<void*>(&k_adj_window<C, KX, KY, TAPS_AA, 128>)
-                         : reinterpret_cast<void*>(&k_adj_window<C, KX, KY, TAPS_AA>);
+    if (tm == TAPS_AA) return reinterpret_cast<void*>(&k_adj_window<C, KX, KY, TAPS_AA>);
     return reinterpret_cast<void*>(&k_adj_window<C, KX, KY, TAPS_TABLE>);
 }
 
 template <int C, int KX>
-static void* adj_window_fy(int KY, int tm, int nt)
+static void* adj_window_fy(int KY, int tm)
 {
-    return KY == 2 ? adj_window_func<C, KX, 2>(tm, nt) : KY == 4 ? adj_window_func<C, KX, 4>(tm, nt)
-                                                               : adj_window_func<C, KX, 8>(tm, nt);
+    return KY == 2 ? adj_window_func<C, KX, 2>(tm) : KY == 4 ? adj_window_func<C, KX, 4>(tm) : adj_window_func<C, KX, 8>(tm);
 }
 
 template <int C>
-static void* adj_window_fx(int KX, int KY, int tm, int nt)
+static void* adj_window_fx(int KX, int KY, int tm)
 {
-    if (tm == TAPS_POINT) {   // the method's own taps on both axes: KX == KY in {2, 4}
-        if (nt == 128)
-            return KX == 2 ? reinterpret_cast<void*>(&k_adj_window<C, 2, 2, TAPS_POINT, 128>)
-                           : reinterpret_cast<void*>(&k_adj_window<C, 4, 4, TAPS_POINT, 128>);
+    if (tm == TAPS_POINT)   // the method's own taps on both axes: KX == KY in {2, 4}
         return KX == 2 ? reinterpret_cast<void*>(&k_adj_window<C, 2, 2, TAPS_POINT>)
                        : reinterpret_cast<void*>(&k_adj_window<C, 4, 4, TAPS_POINT>);
-    }
-    return KX == 2 ? adj_window_fy<C, 2>(KY, tm, nt) : KX == 4 ? adj_window_fy<C, 4>(KY, tm, nt)
-                                                               : adj_window_fy<C, 8>(KY, tm, nt);
+    return KX == 2 ? adj_window_fy<C, 2>(KY, tm) : KX == 4 ? adj_window_fy<C, 4>(KY, tm) : adj_window_fy<C, 8>(KY, tm);
 }
 
 static cudaError_t launch_adj_window(const Geom& g, const BwdPlan& p, const float* dY, float* dX, const AdjTables& tb,
@@ -1068,9 +1064,9 @@ static cudaError_t launch_adj_window(const Geom& g, const BwdPlan& p, const floa
 {
     const int KX = adj_taps_class(p.xK), KY = adj_taps_class(p.yK);
     if (tm == TAPS_POINT && (KX != KY || KX > 4)) return cudaErrorInvalidValue;
-    if (c.nt != kAwThreads && (c.nt != 128 || tm == TAPS_TABLE)) return cudaErrorInvalidValue;
-    void* func = g.C == 1 ? adj_window_fx<1>(KX, KY, tm, c.nt) : g.C == 2 ? adj_window_fx<2>(KX, KY, tm, c.nt)
-               : g.C == 3 ? adj_window_fx<3>(KX, KY, tm, c.nt) : adj_window_fx<4>(KX, KY, tm, c.nt);
+    if (c.nt < 32 || c.nt > kAwThreads || c.nt % 32) return cudaErrorInvalidValue;
+    void* func = g.C == 1 ? adj_window_fx<1>(KX, KY, tm) : g.C == 2 ? adj_window_fx<2>(KX, KY, tm)
+               : g.C == 3 ? adj_window_fx<3>(KX, KY, tm) : adj_window_fx<4>(KX, KY, tm);
     int per_sm = 1;
     cudaError_t e = prepare_kernel(func, c.smem, c.nt, &per_sm);
     if (e != cudaSuccess) return e;

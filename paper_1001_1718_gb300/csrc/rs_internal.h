@@ -115,7 +115,7 @@ struct StreamCfg {
 };
 
 // Configuration of the register-window kernel (bilinear / bicubic): strips
-// of kWinThreads * P output pixels (P per thread, win_pixels), bands of
+// of nt * P output pixels (P per thread, win_pixels), bands of
 // band_h output rows (0 = from occupancy and `waves`), source rows staged
 // in chunks of `chunk` rows (a multiple of the taps). The rest are
 // host-computed bounds every block checks its own strip and band against
@@ -131,7 +131,7 @@ struct WinCfg {
     int aa_method;   // antialias taps: M_BILINEAR / M_BICUBIC (the stretched kernel)
     int strip;       // antialias taps: output pixels per block (at most the kernel's 128 P)
     int pat;         // uint8 sources read in place (win_raw.cuh): the ratio range + 1 (0: the other forms)
-    int nt;          // ditto: threads per block
+    int nt;          // threads per block (128 in the antialias and batch kernels)
     size_t smem;
 };
 

@@ -115,7 +115,9 @@ bool win_config(const Geom& g, int method, int dtype, WinCfg& c, bool allow_x2)
     const int es = (int)dtype_size(dtype);
     const bool x2 = allow_x2 && win_is_x2(g);
     const int P = win_pixels(g.C, dtype, x2);
-    const int SP = kWinThreads * P;
+    // narrow rows: only the warps they fill (the batch's blocks are all alike)
+    c.nt = allow_x2 ? win_raw_threads(g.Wo, 32 * P) : kWinThreads;
+    const int SP = c.nt * P;
     c.pat = 0;
     // source pixels a strip's footprint can span
     const int span_px = tap_span_bound(SP, g.W, g.Wo, KT, g.coord);
@@ -125,7 +127,7 @@ bool win_config(const Geom& g, int method, int dtype, WinCfg& c, bool allow_x2)
         const int half = P / 2 * g.C;
         const int fpl = (P / 2 + KT - 1) * g.C;
         const int nf = (fpl * es + 3) / 4, nr = es == 4 ? nf : nf + 1;
-        const int need = std::max(per * 16, 16 + (kWinThreads - 1) * half * es + 4 * nr);
+        const int need = std::max(per * 16, 16 + (c.nt - 1) * half * es + 4 * nr);
         c.swe = 0;
         c.raw_row = (need + 15) & ~15;
     } else {    // channel-planar FP32 rows and a two-slot raw ring
@@ -220,9 +222,9 @@ cudaError_t launch_win(const Geom& g, int method, int dtype, const void* src, vo
     void* func = win_kernel(method, dtype, g.C, x2);
     if (!func) return cudaErrorInvalidValue;
     int per_sm = 1;
-    cudaError_t e = prepare_kernel(func, c.smem, kWinThreads, c.band_h <= 0 ? &per_sm : nullptr);
+    cudaError_t e = prepare_kernel(func, c.smem, c.nt, c.band_h <= 0 ? &per_sm : nullptr);
     if (e != cudaSuccess) return e;
-    const int SP = kWinThreads * win_pixels(g.C, dtype, x2);
+    const int SP = c.nt * win_pixels(g.C, dtype, x2);
     const int64_t strips = ((int64_t)g.Wo + SP - 1) / SP;
     if (c.band_h <= 0) {
         const int64_t resident = (int64_t)num_sms() * std::max(1, per_sm);
@@ -239,7 +241,7 @@ cudaError_t launch_win(const Geom& g, int method, int dtype, const void* src, vo
     dim3 grid((unsigned)strips, (unsigned)((g.Ho + c.band_h - 1) / c.band_h), (unsigned)g.planes);
     unsigned int* fw = fault_word();
     void* args[] = {const_cast<Geom*>(&g), const_cast<void**>(&src), &dst, &c, &fw};
-    e = cudaLaunchKernel(func, grid, dim3(kWinThreads), args, c.smem, st);
+    e = cudaLaunchKernel(func, grid, dim3(c.nt), args, c.smem, st);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 

@@ -1,7 +1,7 @@
 // Register-window resampling (bilinear / bicubic): the per-block work of the
 // forward window kernel and of the batch's window items.
 //
-// A block of kWinThreads threads owns a strip of SP = kWinThreads * P output
+// A block of NT (at most kWinThreads) threads owns a strip of NT P output
 // pixels (all C channels) and a band of output rows; each thread owns P
 // pixels of the strip for the whole band.
 //
@@ -51,7 +51,6 @@
 namespace rs {
 
 static constexpr int kWinThreads = 128;
-static constexpr int kWinWarps = kWinThreads / 32;
 static constexpr int kWinMaxBand = 256;   // rows of the per-block row-tap tables
 
 template <int C, typename T, bool X2>
@@ -63,7 +62,6 @@ struct WinShape {
                                 : (C == 1 ? 8 : C == 4 ? 2 : 4);
     static constexpr int NP = P / 2;                 // pixel pairs
     static constexpr int E = P * C;                  // elements per thread per row
-    static constexpr int SP = kWinThreads * P;       // strip width in pixels
     // X2 run: bytes, 32-bit words and widest store unit per output row; the
     // staged floats between consecutive threads' footprints and the vector
     // width (floats) of their footprint loads.
@@ -286,7 +284,6 @@ template <int C, typename T, int TM, int KT>
 struct WinGen {
     static constexpr int P0 = WinShape<C, T, false>::P;
     static constexpr int P = (TM == TAP_AA && KT > 4) ? (P0 / 2 < 2 ? 2 : P0 / 2) : P0;
-    static constexpr int SP = kWinThreads * P;
 };
 
 template <int KT, int C, typename T, typename TO = T, bool NORM = false, int TM = TAP_POINT>
@@ -294,14 +291,15 @@ __device__ __forceinline__ void win_body(const Geom& g, const T* __restrict__ s,
                                          int bx, int by, float* sm, unsigned int* fault, const NormOut& no = NormOut{})
 {
     using S = WinGen<C, T, TM, KT>;
-    constexpr int P = S::P, NP = P / 2, NT = kWinThreads;
+    constexpr int P = S::P, NP = P / 2;
     constexpr int ES = (int)sizeof(T);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int NT = blockDim.x;   // fewer than kWinThreads where the rows are narrow
 
-    // Strip of output pixels: 128 P, or for antialias taps cfg.strip <= 128 P
+    // Strip of output pixels: P per thread, or for antialias taps cfg.strip <= 128 P
     // (a narrower strip keeps a large downscale's footprint in shared memory;
     // the lanes past it idle in the arithmetic and still stage rows).
-    const int sw_px = TM == TAP_AA ? cfg.strip : S::SP;
+    const int sw_px = TM == TAP_AA ? cfg.strip : NT * P;
     const int j_lo = bx * sw_px;                     // first pixel of the strip
     const int j_hi = min(g.Wo, j_lo + sw_px) - 1;    // last pixel of the strip
     const int yb = by * cfg.band_h;
@@ -440,7 +438,7 @@ __device__ __forceinline__ void win_body(const Geom& g, const T* __restrict__ s,
     auto convert = [&](int c) {
         const int r0 = r_first + c * R, nn = chunk_rows(c);
         const unsigned char* rbase = RAW + (size_t)(c & 1) * R * cfg.raw_row;
-        for (int k = warp; k < nn; k += kWinWarps) {
+        for (int k = warp; k < nn; k += NT >> 5) {
             const int phase = (int)(reinterpret_cast<uintptr_t>(row_ptr(r0 + k)) & 15);
             const unsigned char* rrow = rbase + k * cfg.raw_row;
             float* dr = SR + k * cfg.swe;
@@ -634,7 +632,8 @@ __device__ __forceinline__ void win_body_x2(const Geom& g, const T* __restrict__
                                             const NormOut& no = NormOut{})
 {
     using S = WinShape<C, T, true>;
-    constexpr int P = S::P, NP = S::NP, NT = kWinThreads;
+    constexpr int P = S::P, NP = S::NP;
+    const int NT = blockDim.x;   // fewer than kWinThreads where the rows are narrow
     constexpr int ES = (int)sizeof(T);
     constexpr int HK = KT / 2 - 1;              // footprint pixels left of a thread's first source pixel
     constexpr int FPL = (NP + KT - 1) * C;      // footprint elements of a thread
@@ -642,8 +641,8 @@ __device__ __forceinline__ void win_body_x2(const Geom& g, const T* __restrict__
     constexpr int NR = ES == 4 ? NF : NF + 1;   // words read
     const int tid = threadIdx.x;
 
-    const int j_lo = bx * S::SP;
-    const int j_hi = min(g.Wo, j_lo + S::SP) - 1;
+    const int j_lo = bx * NT * P;
+    const int j_hi = min(g.Wo, j_lo + NT * P) - 1;
     const int yb = by * cfg.band_h;
     const int ye = min(g.Ho, yb + cfg.band_h);
     const int nrows = ye - yb;

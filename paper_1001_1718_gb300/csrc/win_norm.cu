@@ -72,9 +72,9 @@ cudaError_t launch_win_norm(const Geom& g, int method, int out_dtype, const void
     void* func = x2 ? win_norm_kernel_x2(method, out_dtype, g.C) : norm_kernel_part(method, out_dtype, g.C);
     if (!func) return cudaErrorInvalidValue;
     int per_sm = 1;
-    cudaError_t e = prepare_kernel(func, c.smem, kWinThreads, c.band_h <= 0 ? &per_sm : nullptr);
+    cudaError_t e = prepare_kernel(func, c.smem, c.nt, c.band_h <= 0 ? &per_sm : nullptr);
     if (e != cudaSuccess) return e;
-    const int SP = kWinThreads * win_pixels(g.C, DT_U8, x2);
+    const int SP = c.nt * win_pixels(g.C, DT_U8, x2);
     const int64_t strips = ((int64_t)g.Wo + SP - 1) / SP;
     if (c.band_h <= 0) {
         const int64_t resident = (int64_t)num_sms() * std::max(1, per_sm);
@@ -87,7 +87,7 @@ cudaError_t launch_win_norm(const Geom& g, int method, int out_dtype, const void
     dim3 grid((unsigned)strips, (unsigned)((g.Ho + c.band_h - 1) / c.band_h), (unsigned)g.planes);
     unsigned int* fw = fault_word();
     void* args[] = {const_cast<Geom*>(&g), const_cast<void**>(&src), &dst, &c, const_cast<NormOut*>(&no), &fw};
-    e = cudaLaunchKernel(func, grid, dim3(kWinThreads), args, c.smem, st);
+    e = cudaLaunchKernel(func, grid, dim3(c.nt), args, c.smem, st);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 #endif
