@@ -160,8 +160,14 @@ static bool default_choice(const Geom& g, int method, int dtype, const void* src
         }
     }
     if ((g.Ho >= g.H || dtype == DT_U8) && out_elems >= (int64_t)1 << 22) {
+        // Large float outputs of the exact-x2 form (bound by HBM) in five blocks
+        // per slot: their stores start and end evenly (bicubic, two / five:
+        // FP32 4096^2 -> 8192^2 61.6 / 54.2 us, FP16 8192^2 -> 16384^2 116 /
+        // 110); below ~192 MB of output the extra prologues cost more
+        // (BF16 4096^2, 128 MB: 33.3 / 37.3).
+        const bool big_x2 = dtype != DT_U8 && win_is_x2(g) && out_elems * (int64_t)dtype_size(dtype) >= (int64_t)192 << 20;
         for (int ch : {8, 4}) {
-            const Tuned t{RS_IMPL_WINDOW, 1024, ch, 128, g.Ho < g.H && g.planes == 1 ? 1 : 2};
+            const Tuned t{RS_IMPL_WINDOW, 1024, ch, 128, g.Ho < g.H && g.planes == 1 ? 1 : big_x2 ? 5 : 2};
             if (make_choice(g, method, dtype, src, t, k) && k.window.smem <= (ch == 8 ? 56 : 100) * 1024) return true;
         }
     }
