@@ -179,24 +179,20 @@ def resize(x: torch.Tensor, size: Sequence[int], method="bilinear", *, layout: s
     a, threads, waves, antialias = float(cubic_a), int(threads), int(waves), bool(antialias)
     tw, th = (tile or (0, 0))
     tile = (int(tw), int(th))
-    key = call = None
-    if out is None:
-        key = ("resize", x.shape, x.stride(), x.dtype, Ho, Wo, _code(METHODS, method, "method"), layout,
-               _code(COORDS, coord, "coord"), a, _code(IMPLS, impl, "impl"), tile, threads, waves, antialias)
-        call = _CALLS.get(key)
+    if out is not None:
+        _require_cuda(out)
+        if out.dtype != x.dtype:
+            raise ValueError("out must have the dtype of x")
+    key = ("resize", x.shape, x.stride(), x.dtype, Ho, Wo, _code(METHODS, method, "method"), layout,
+           _code(COORDS, coord, "coord"), a, _code(IMPLS, impl, "impl"), tile, threads, waves, antialias,
+           out is not None and (out.shape, out.stride()))
+    call = _CALLS.get(key)
     if call is None:
         shape = _out_shape(x, layout, Ho, Wo)
-        if out is None:
-            Lo = _dense_layout(shape, layout)
-        else:
-            _require_cuda(out)
-            if out.dtype != x.dtype:
-                raise ValueError("out must have the dtype of x")
-            Lo = _layout(out, layout)
+        Lo = _dense_layout(shape, layout) if out is None else _layout(out, layout)
         call = (shape, ctypes.byref(_layout(x, layout)), ctypes.byref(Lo), _dtype(x),
                 _code(METHODS, method, "method"), ctypes.byref(_opts(coord, a, impl, tile, threads, waves, antialias)))
-        if key is not None:
-            _remember(key, call)
+        _remember(key, call)
     shape, Li, Lo, dt, m, o = call
     if out is None:
         out = torch.empty(shape, dtype=x.dtype, device=x.device)
@@ -227,11 +223,10 @@ def resize_normalize(x: torch.Tensor, size: Sequence[int], method="bilinear", me
     Ho, Wo = int(size[0]), int(size[1])
     a, chunk, antialias = float(cubic_a), int(chunk), bool(antialias)
     mean, std = tuple(float(v) for v in mean), tuple(float(v) for v in std)
-    key = call = None
-    if out is None:
-        key = ("normalize", x.shape, x.stride(), odt, Ho, Wo, _code(METHODS, method, "method"), mean, std,
-               _code(COORDS, coord, "coord"), a, _code(IMPLS, impl, "impl"), chunk, antialias)
-        call = _CALLS.get(key)
+    key = ("normalize", x.shape, x.stride(), odt, Ho, Wo, _code(METHODS, method, "method"), mean, std,
+           _code(COORDS, coord, "coord"), a, _code(IMPLS, impl, "impl"), chunk, antialias,
+           out is not None and (out.shape, out.stride(), out.dtype))
+    call = _CALLS.get(key)
     if call is None:
         batched = x.dim() == 4
         C = x.shape[-1]
@@ -248,8 +243,7 @@ def resize_normalize(x: torch.Tensor, size: Sequence[int], method="bilinear", me
         call = (shape, ctypes.byref(Li), ctypes.byref(Lo), _code(METHODS, method, "method"),
                 (ctypes.c_float * C)(*mean), (ctypes.c_float * C)(*std),
                 ctypes.byref(_opts(coord, a, impl, (0, chunk), 0, 0, antialias)))
-        if key is not None:
-            _remember(key, call)
+        _remember(key, call)
     shape, Li, Lo, m, cm, cs, o = call
     if out is None:
         out = torch.empty(shape, dtype=dtype, device=x.device)
@@ -282,11 +276,10 @@ def resize_backward(grad_out: torch.Tensor, in_hw, method="bilinear", *, layout:
     _require_cuda(grad_out)
     H, W = int(in_hw[0]), int(in_hw[1])
     a, antialias = float(cubic_a), bool(antialias)
-    key = call = None
-    if grad_in is None:
-        key = ("backward", grad_out.shape, grad_out.stride(), grad_out.dtype, H, W, _code(METHODS, method, "method"),
-               layout, _code(COORDS, coord, "coord"), a, _code(IMPLS, impl, "impl"), antialias)
-        call = _CALLS.get(key)
+    key = ("backward", grad_out.shape, grad_out.stride(), grad_out.dtype, H, W, _code(METHODS, method, "method"),
+           layout, _code(COORDS, coord, "coord"), a, _code(IMPLS, impl, "impl"), antialias,
+           grad_in is not None and (grad_in.shape, grad_in.stride()))
+    call = _CALLS.get(key)
     if call is None:
         shape = _out_shape(grad_out, layout, H, W)
         Lo = ctypes.byref(_layout(grad_out, layout))
@@ -296,8 +289,7 @@ def resize_backward(grad_out: torch.Tensor, in_hw, method="bilinear", *, layout:
         n = ctypes.c_size_t(0)
         B.check(lib().rs_resize_backward_workspace(Lo, Li, m, o, ctypes.byref(n)), "rs_resize_backward_workspace")
         call = (shape, Lo, Li, _dtype(grad_out), m, o, n.value)
-        if key is not None:
-            _remember(key, call)
+        _remember(key, call)
     shape, Lo, Li, dt, m, o, nbytes = call
     if grad_in is None:
         grad_in = torch.empty(shape, dtype=grad_out.dtype, device=grad_out.device)

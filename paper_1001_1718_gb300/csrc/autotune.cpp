@@ -116,10 +116,10 @@ static bool make_choice(const Geom& g, int method, int dtype, const void* src, c
         k.window.chunk = t.tile_h;
         k.window.waves = t.waves;
         if (!win_config(g, method, dtype, k.window)) return false;
-        // uint8 sources with at most two source pixels per output pixel along
+        // uint8 sources with at most three source pixels per output pixel along
         // x: the form that reads them in place
         WinCfg raw = k.window;
-        if (win_raw_config(g, method, dtype, win_raw_threads(g.Wo, 124), 256, raw)) k.window = raw;
+        if (win_raw_config(g, method, dtype, win_raw_block(g, 124), 256, raw)) k.window = raw;
         return true;
     }
     if (t.impl == RS_IMPL_REDUCE) return reduce_config(g, method, dtype, src, nullptr);

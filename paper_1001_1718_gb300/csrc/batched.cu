@@ -410,7 +410,7 @@ static rs_status prepare_image(const rs_image_desc& x, int dtype, const rs_optio
             raw.chunk = sh.chunk;
             // a downscale's output row takes several source rows: shorter bands
             const int band = x.Ho < x.H ? std::max(std::min(sh.band, kHeavyBand), (int)((int64_t)sh.band * x.Ho / x.H)) : sh.band;
-            if (win_raw_default(g, x.method, dtype, kRawThreads, band, raw, false)) {   // uint8 read in place
+            if (win_raw_default(g, x.method, dtype, kRawThreads, band, raw, false) && raw.pat <= 3) {   // uint8 read in place, up to 2 source pixels per output pixel
                 im.kind = 3;
                 im.pat = raw.pat;
                 im.chunk = raw.chunk;

@@ -242,11 +242,12 @@ rs_status rs_resize_normalize(const void* src, const rs_layout* in, void* dst, c
         }
     }
     if (!ok) return o.tile_h ? RS_ERR_INVALID_ARG : RS_ERR_UNSUPPORTED;
-    // grey and RGB sources, at most two source pixels per output pixel along
+    // grey and RGB sources, at most three source pixels per output pixel along
     // x: the form that reads the source in place
     WinCfg raw = c;
     raw.chunk = o.tile_h;
-    if ((g.C == 1 || g.C == 3) && win_raw_default(g, method, DT_U8, win_raw_threads(g.Wo, 128), 256, raw))
+    if ((g.C == 1 || g.C == 3) && win_raw_default(g, method, DT_U8, win_raw_block(g, 128), 256, raw) &&
+        win_raw_norm_ok(g, dst, raw, no))
         return cuda_status(launch_win_raw_norm(g, method, src, dst, raw, no, static_cast<cudaStream_t>(stream)));
     return cuda_status(launch_win_norm(g, method, out_dtype, src, dst, c, no, static_cast<cudaStream_t>(stream)));
 }

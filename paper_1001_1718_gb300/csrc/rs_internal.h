@@ -205,14 +205,17 @@ bool win_is_x2(const Geom& g);
 bool win_config(const Geom& g, int method, int dtype, WinCfg& c, bool allow_x2 = true);
 // The form that reads uint8 sources in place (win_raw.cuh): configuration for
 // blocks of nt threads and bands of at most band_cap rows (false where it does
-// not apply: other dtypes, more than two source pixels per output pixel along
-// x), its default (c.chunk 0: 8 staged rows at a time, or 4 where 8 leave no
+// not apply: other dtypes, more than three source pixels per output pixel
+// along x), its default (c.chunk 0: 8 staged rows at a time, or 4 where 8 leave no
 // room for four blocks per SM) and launches (band_h 0 = from occupancy and
 // waves).
 bool win_raw_config(const Geom& g, int method, int dtype, int nt, int band_cap, WinCfg& c, bool allow_x2 = true);
 bool win_raw_default(const Geom& g, int method, int dtype, int nt, int band_cap, WinCfg& c, bool allow_x2 = true);
 int win_raw_threads(int Wo, int warp_px);
+int win_raw_block(const Geom& g, int warp_px);   // its threads per block for a problem
 cudaError_t launch_win_raw(const Geom& g, int method, const void* src, void* dst, WinCfg c, cudaStream_t st);
+// Whether the pre-process's output rows suit the form (win_raw.cu).
+bool win_raw_norm_ok(const Geom& g, const void* dst, const WinCfg& c, const NormOut& no);
 cudaError_t launch_win_raw_norm(const Geom& g, int method, const void* src, void* dst, WinCfg c, const NormOut& no,
                                 cudaStream_t st);
 cudaError_t launch_win(const Geom& g, int method, int dtype, const void* src, void* dst, WinCfg c, cudaStream_t st);

@@ -115,8 +115,10 @@ bool win_config(const Geom& g, int method, int dtype, WinCfg& c, bool allow_x2)
     const int es = (int)dtype_size(dtype);
     const bool x2 = allow_x2 && win_is_x2(g);
     const int P = win_pixels(g.C, dtype, x2);
-    // narrow rows: only the warps they fill (the batch's blocks are all alike)
-    c.nt = allow_x2 ? win_raw_threads(g.Wo, 32 * P) : kWinThreads;
+    // narrow rows: only the warps they fill (the batch's blocks are all alike;
+    // a downscale's block spends most of its time staging rows, which idle
+    // lanes share)
+    c.nt = allow_x2 && g.Wo >= g.W ? win_raw_threads(g.Wo, 32 * P) : kWinThreads;
     const int SP = c.nt * P;
     c.pat = 0;
     // source pixels a strip's footprint can span

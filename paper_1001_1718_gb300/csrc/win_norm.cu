@@ -42,14 +42,11 @@ template <int KT, typename TO>
 static void* norm_func_c(int C)
 {
     switch (C) {
-#if WIN_NORM_PART == 0   // (exact x2 of 1 and 3 channels: win_raw.cu)
     case 1: return norm_func<KT, 1, TO>();
-    case 3: return norm_func<KT, 3, TO>();
-#endif
     case 2: return norm_func<KT, 2, TO>();
-    case 4: return norm_func<KT, 4, TO>();
+    case 3: return norm_func<KT, 3, TO>();
+    default: return norm_func<KT, 4, TO>();
     }
-    return nullptr;
 }
 
 static void* norm_kernel_part(int method, int out_dtype, int C)
@@ -70,7 +67,6 @@ cudaError_t launch_win_norm(const Geom& g, int method, int out_dtype, const void
 {
     const bool x2 = win_is_x2(g);
     void* func = x2 ? win_norm_kernel_x2(method, out_dtype, g.C) : norm_kernel_part(method, out_dtype, g.C);
-    if (!func) return cudaErrorInvalidValue;
     int per_sm = 1;
     cudaError_t e = prepare_kernel(func, c.smem, c.nt, c.band_h <= 0 ? &per_sm : nullptr);
     if (e != cudaSuccess) return e;

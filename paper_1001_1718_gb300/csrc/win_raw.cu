@@ -24,7 +24,7 @@ namespace rs {
 // 58.2, three: 60.6; the form on FP32 windows it replaces: 77.9).
 // Four channels of whole bicubic runs need a few registers more.
 template <int KT, int C, int PAT, int ST>
-constexpr int raw_blocks() { return (PAT == kRawX2 ? 5 : 4) - (KT == 4 && C == 4 && ST == RAW_WORDS); }
+constexpr int raw_blocks() { return (PAT == kRawX2 ? 5 : PAT == 4 && KT == 4 && C > 2 ? 3 : 4) - (KT == 4 && C == 4 && ST == RAW_WORDS && PAT < 4); }
 
 template <int KT, int C, int PAT, int ST>
 __global__ void __launch_bounds__(kWinThreads, raw_blocks<KT, C, PAT, ST>())
@@ -56,16 +56,24 @@ static void* raw_func_s(int st)
     return st == RAW_WORDS ? (void*)&k_win_raw<kRawKT, C, PAT, RAW_WORDS> : (void*)&k_win_raw<kRawKT, C, PAT, RAW_ANY>;
 }
 
-// FP32 outputs leave element by element at any alignment.
+// The fused pre-process: whole aligned runs, and for downscales (whose gain
+// is the footprint) any alignment too: a thread's elements leave one by one
+// there, 8 to 16 bytes apart in a warp, which costs upscales more than the
+// form gains (9 x 1068 x 1171 -> 1473 x 1615 BF16 bicubic: 98 us, the general
+// form's stores of neighbouring pixels 94).
+template <int C, int PAT, typename TO>
+static void* norm_func_t(int st)
+{
+    if (st == RAW_WORDS) return (void*)&k_win_raw_norm<kRawKT, C, PAT, RAW_WORDS, TO>;
+    if constexpr (PAT == 2 || PAT == 4) return (void*)&k_win_raw_norm<kRawKT, C, PAT, RAW_ANY, TO>;
+    return nullptr;
+}
+
 template <int C, int PAT>
 static void* norm_func_s(int st, int out_dtype)
 {
-    if (out_dtype == DT_F32) return (void*)&k_win_raw_norm<kRawKT, C, PAT, RAW_ANY, float>;
-    if (out_dtype == DT_F16)
-        return st == RAW_WORDS ? (void*)&k_win_raw_norm<kRawKT, C, PAT, RAW_WORDS, __half>
-                               : (void*)&k_win_raw_norm<kRawKT, C, PAT, RAW_ANY, __half>;
-    return st == RAW_WORDS ? (void*)&k_win_raw_norm<kRawKT, C, PAT, RAW_WORDS, __nv_bfloat16>
-                           : (void*)&k_win_raw_norm<kRawKT, C, PAT, RAW_ANY, __nv_bfloat16>;
+    return out_dtype == DT_F32 ? norm_func_t<C, PAT, float>(st) : out_dtype == DT_F16 ? norm_func_t<C, PAT, __half>(st)
+                               : norm_func_t<C, PAT, __nv_bfloat16>(st);
 }
 
 template <int C>
@@ -74,10 +82,11 @@ static void* raw_func_p(int pat, int st, int out_dtype)
 #if WIN_RAW_PART < 2
     (void)out_dtype;
     return pat == 0 ? raw_func_s<C, 0>(st) : pat == 1 ? raw_func_s<C, 1>(st) : pat == 2 ? raw_func_s<C, 2>(st)
-                                                                             : raw_func_s<C, kRawX2>(st);
+         : pat == 4 ? raw_func_s<C, 4>(st) : raw_func_s<C, kRawX2>(st);
 #else
     return pat == 0 ? norm_func_s<C, 0>(st, out_dtype) : pat == 1 ? norm_func_s<C, 1>(st, out_dtype)
-         : pat == 2 ? norm_func_s<C, 2>(st, out_dtype) : norm_func_s<C, kRawX2>(st, out_dtype);
+         : pat == 2 ? norm_func_s<C, 2>(st, out_dtype) : pat == 4 ? norm_func_s<C, 4>(st, out_dtype)
+                                                                  : norm_func_s<C, kRawX2>(st, out_dtype);
 #endif
 }
 
@@ -121,6 +130,14 @@ int win_raw_threads(int Wo, int warp_px)
     return 32 * best;
 }
 
+// Strips of half the width beyond two source pixels per output pixel: their
+// staged rows are as long as a full strip's at half the ratio.
+int win_raw_block(const Geom& g, int warp_px)
+{
+    const int nt = win_raw_threads(g.Wo, warp_px);
+    return (int64_t)g.W > 2 * (int64_t)g.Wo ? std::min(nt, 64) : nt;
+}
+
 bool win_raw_config(const Geom& g, int method, int dtype, int nt, int band_cap, WinCfg& c, bool allow_x2)
 {
     c.pat = 0;
@@ -133,7 +150,8 @@ bool win_raw_config(const Geom& g, int method, int dtype, int nt, int band_cap, 
     if (pat < 0) return false;
     const int span = tap_span_bound(kRawP * nt, g.W, g.Wo, KT, g.coord) * g.C;
     const int fw = (pat == 0 ? RawPat<0>::hi(kRawP - 1) : pat == 1 ? RawPat<1>::hi(kRawP - 1)
-                    : pat == 2 ? RawPat<2>::hi(kRawP - 1) : RawPat<kRawX2>::hi(kRawP - 1)) + KT;
+                    : pat == 2 ? RawPat<2>::hi(kRawP - 1) : pat == 4 ? RawPat<4>::hi(kRawP - 1)
+                    : RawPat<kRawX2>::hi(kRawP - 1)) + KT;
     const int nr = (fw * g.C + 3) / 4 + 1;   // words a thread reads of a row
     c.nt = nt;
     c.raw_row = std::max((span + 15) / 16 + 2, (15 + span + 4 * nr + 15) / 16) * 16;
@@ -212,11 +230,20 @@ cudaError_t launch_win_raw(const Geom& g, int method, const void* src, void* dst
     return launch_raw(g, func, raw_strip(c.nt, raw_overlap(mode, 1)), src, dst, c, nullptr, st);
 }
 
+bool win_raw_norm_ok(const Geom& g, const void* dst, const WinCfg& c, const NormOut& no)
+{
+    // three FP32 planes of an exact x2 are all stores: the form on consecutive
+    // pairs keeps them a little faster (16 x 512^2 bicubic 38 us, here 39.5)
+    if (c.pat == kRawX2 + 1 && no.dtype == DT_F32 && g.C == 3) return false;
+    const size_t es = dtype_size(no.dtype);
+    return c.pat == 2 + 1 || c.pat == 4 + 1 || raw_store_mode(g, dst, es, kRawP * (int)es, no.c_stride) == RAW_WORDS;
+}
+
 cudaError_t launch_win_raw_norm(const Geom& g, int method, const void* src, void* dst, WinCfg c, const NormOut& no,
                                 cudaStream_t st)
 {
     const size_t es = dtype_size(no.dtype);
-    const int mode = no.dtype == DT_F32 ? RAW_ANY : raw_store_mode(g, dst, es, 8, no.c_stride);
+    const int mode = raw_store_mode(g, dst, es, kRawP * (int)es, no.c_stride);
     void* func = method == M_BILINEAR ? raw_norm_bilinear(g.C, c.pat - 1, mode, no.dtype)
                                       : raw_norm_bicubic(g.C, c.pat - 1, mode, no.dtype);
     return launch_raw(g, func, raw_strip(c.nt, raw_overlap(mode, es)), src, dst, c, &no, st);

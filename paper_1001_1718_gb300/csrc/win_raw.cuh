@@ -1,5 +1,5 @@
 // Register-window resampling of uint8 sources read in place: the general
-// form (any vertical ratio, horizontally at most two source pixels per
+// form (any vertical ratio, horizontally at most three source pixels per
 // output pixel) of the forward window kernel, the fused pre-process and the
 // batch's window items.
 //
@@ -22,7 +22,7 @@
 // a sum of finite terms leaves it as it is, so every sum equals the general
 // form's, in the same order, up to the sign of a zero (uint8 samples are
 // always finite; the float dtypes keep win_body, where 0 * inf would not be
-// 0). The ranges are compiled for three ratio ranges (RawPat).
+// 0). The ranges are compiled for four ratio ranges (RawPat).
 //
 // What bounds it: instruction issue (about 36 per output pixel and thread at
 // RGB bicubic x1.7, ALU and FMA pipes at ~45% each, 65% of the issue slots
@@ -43,30 +43,30 @@ namespace rs {
 static constexpr int kRawP = 4;   // output pixels per thread
 
 // Ratio ranges: first-tap offsets [lo(k), hi(k)] of pixel k against pixel 0.
-// PAT 0: r <= 1/2, 1: 1/2 < r <= 1, 2: 1 < r <= 2. PAT 3 is the exact x2 form
-// (the asymmetric map, both axes exactly doubled): pixel 2u and row 2u have
-// t = 0 and are the source samples and window rows themselves, pixel 2u + 1
-// and row 2u + 1 have t = 1/2 and the same weights for every u. A position
-// yields two output rows, there are no row tables, and runs start at even
-// pixels, bands at even rows.
+// PAT 0: r <= 1/2, 1: 1/2 < r <= 1, 2: 1 < r <= 2, 4: 2 < r <= 3. PAT 3 is the
+// exact x2 form (the asymmetric map, both axes exactly doubled): pixel 2u and
+// row 2u have t = 0 and are the source samples and window rows themselves,
+// pixel 2u + 1 and row 2u + 1 have t = 1/2 and the same weights for every u. A
+// position yields two output rows, there are no row tables, and runs start at
+// even pixels, bands at even rows.
 static constexpr int kRawX2 = 3;
 template <int PAT>
 struct RawPat {
     static __host__ __device__ constexpr int lo(int k)
     {
-        return PAT == 0 ? 0 : PAT == 1 ? (k < 2 ? 0 : 1) : PAT == 2 ? k : k >> 1;
+        return PAT == 0 ? 0 : PAT == 1 ? (k < 2 ? 0 : 1) : PAT == 2 ? k : PAT == 4 ? 2 * k : k >> 1;
     }
     static __host__ __device__ constexpr int hi(int k)
     {
-        return PAT == 0 ? (k == 0 ? 0 : k < 3 ? 1 : 2) : PAT == 1 ? k : PAT == 2 ? 2 * k : k >> 1;
+        return PAT == 0 ? (k == 0 ? 0 : k < 3 ? 1 : 2) : PAT == 1 ? k : PAT == 2 ? 2 * k : PAT == 4 ? 3 * k : k >> 1;
     }
 };
 
 // The ratio range of an axis advancing an / am source pixels per output
-// pixel, or -1 beyond 2.
+// pixel, or -1 beyond 3.
 inline __host__ __device__ int raw_pattern(int64_t an, int64_t am)
 {
-    return 2 * an <= am ? 0 : an <= am ? 1 : an <= 2 * am ? 2 : -1;
+    return 2 * an <= am ? 0 : an <= am ? 1 : an <= 2 * am ? 2 : an <= 3 * am ? 4 : -1;
 }
 
 // Source pixels of a thread's footprint, and the words read for it.

@@ -25,7 +25,9 @@ def check(H, W, C, Ho, Wo, method, coord, a=-0.5, pad=0, off=0):
     buf, y = image(7, Ho, Wo, C, pad, off)
     before = buf.clone()
     ref = rs.resize(x.contiguous(), (Ho, Wo), method, coord=coord, cubic_a=a, impl="tiled")
-    rs.resize(x, (Ho, Wo), method, coord=coord, cubic_a=a, impl="window", out=y)
+    # (beyond two source pixels per output pixel the default chunk of 8 rows is
+    # refused: the general form's footprint rule)
+    rs.resize(x, (Ho, Wo), method, coord=coord, cubic_a=a, impl="window", tile=(0, 4) if W > 2 * Wo else None, out=y)
     assert rs.debug_fault() == 0
     assert torch.equal(y, ref)
     y.copy_(before[off:off + Ho * (Wo * C + pad)].view(Ho, Wo * C + pad)[:, :Wo * C].unflatten(1, (Wo, C)))
@@ -43,12 +45,12 @@ def test_widths(Wo, method):
         check(23, W, C, 37, Wo, method, COORDS[(k + 1) % 3], pad=k + 1, off=k + 3)
 
 
-# Ratios at and around the bounds of the three ratio ranges (1/2, 1, 2 source
+# Ratios at and around the bounds of the four ratio ranges (1/2, 1, 2, 3 source
 # pixels per output pixel), and vertical ratios of their own.
 @pytest.mark.parametrize("coord", COORDS)
 @pytest.mark.parametrize("W,Wo", [(100, 401), (100, 400), (150, 449), (200, 400), (201, 401), (200, 399), (256, 384),
                                   (400, 401), (300, 300), (401, 400), (600, 400), (799, 400), (800, 400), (801, 401),
-                                  (1023, 512)])
+                                  (1023, 512), (1025, 512), (1201, 400), (1199, 400), (900, 300)])
 def test_ratios(W, Wo, coord):
     for method, a in (("bilinear", -0.5), ("bicubic", -0.5), ("bicubic", -0.75)):
         for H, Ho in ((37, 90), (90, 37), (1, 5), (5, 1), (300, 300)):
@@ -67,7 +69,7 @@ def test_x2(W, method):
 
 
 @pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16, torch.float32])
-@pytest.mark.parametrize("W,Wo", [(100, 257), (300, 512), (455, 455), (700, 455), (1024, 512), (9, 5), (130, 260), (63, 126)])
+@pytest.mark.parametrize("W,Wo", [(100, 257), (300, 512), (455, 455), (700, 455), (1024, 512), (9, 5), (130, 260), (63, 126), (650, 250), (515, 255)])
 def test_normalize(W, Wo, dtype):
     mean, std = (123.675, 116.28, 103.53), (58.395, 57.12, 57.375)
     for C in (1, 3):
