@@ -44,7 +44,7 @@ BATCH_WORKLOAD = ("batch256_rgb_u8: 256 RGB uint8 images, H, W ~ U{64..2048}, sc
                   "bilinear / bicubic alternating, smooth-field pixels (seed 4)")
 RGB_OPS = (("bicubic_x2", "bicubic", 2.0), ("bicubic_x1.7", "bicubic", 1.7), ("nearest_x2", "nearest", 2.0))
 FALLBACK_HBM_GBS = 6800.0
-KERNEL_NAMES = {"window": "k_win", "stream": "k_stream", "tiled": "k_tiled", "gather": "k_nearest",
+KERNEL_NAMES = {"window": "k_win_raw", "stream": "k_stream", "tiled": "k_tiled", "gather": "k_nearest",
                 "plain": "k_plain"}
 
 
@@ -181,7 +181,8 @@ class ClockSampler:
 # Source files each profiled kernel is built from (a change to any of them
 # voids its recorded DRAM traffic).
 KERNEL_SOURCES = {
-    "k_batched_window": ["batched.cu", "win_body.cuh", "tile_body.cuh", "aa_wide.cuh", "rs_common.cuh", "rs_internal.h"],
+    "k_batched_window": ["batched.cu", "win_raw.cuh", "win_body.cuh", "tile_body.cuh", "aa_wide.cuh", "rs_common.cuh", "rs_internal.h"],
+    "k_win_raw": ["win_raw.cu", "win_raw.cuh", "win_body.cuh", "rs_common.cuh", "rs_internal.h"],
     "k_win": ["win.cu", "win_body.cuh", "rs_common.cuh", "rs_internal.h"],
     "k_stream": ["stream.cu", "rs_common.cuh", "rs_internal.h"],
     "k_tiled": ["tiled.cu", "tile_body.cuh", "rs_common.cuh", "rs_internal.h"],

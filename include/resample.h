@@ -71,22 +71,25 @@ typedef enum { RS_COORD_ASYMMETRIC = 0, RS_COORD_HALF_PIXEL = 1, RS_COORD_ALIGN_
  *          where its footprint fits in shared memory; else STREAM, else
  *          TILED. rs_autotune replaces this choice for a problem it has
  *          timed.
- * WINDOW = bilinear / bicubic, blocks of 128 threads, one per (strip of
- *          output pixels, band of output rows, plane). Source rows are
- *          copied with 16-byte cp.async in chunks of tile_h rows (a
- *          multiple of the taps: 2 bilinear, 4 bicubic) two chunks ahead;
- *          each thread interpolates every source row its pixels' taps reach
- *          horizontally once, keeps the last 2 or 4 such rows in registers,
- *          and blends each output row from them (no shared-memory traffic
- *          per output row). Two forms:
+ * WINDOW = bilinear / bicubic, blocks of up to 128 threads (fewer where the
+ *          rows are narrow), one per (strip of output pixels, band of output
+ *          rows, plane). Source rows are copied with 16-byte cp.async in
+ *          chunks of tile_h rows (a multiple of the taps: 2 bilinear, 4
+ *          bicubic) two chunks ahead; each thread interpolates every source
+ *          row its pixels' taps reach horizontally once, keeps the last 2 or
+ *          4 such rows in registers, and blends each output row from them.
+ *          Forms:
+ *          uint8 up to three source pixels per output pixel along x, any
+ *          vertical ratio: a thread owns 4 consecutive pixels, reads its
+ *          footprint from the copied bytes, sums every pixel over the range
+ *          its taps can take (zero weights at the others) and stores whole
+ *          words at any output alignment;
  *          exact x2 (asymmetric map, both axes exactly doubled): a thread
- *          owns P consecutive output pixels (P * C * size >= 8 bytes where
- *          the row allows), reads its footprint straight from the copied
- *          bytes and stores its run with packed 4- to 16-byte stores; the
- *          even outputs are copies, the odd ones the midpoint weights;
- *          general ratios: a thread owns P pixels 32 apart (strips of
- *          128 P pixels, P = 2 to 8 by channels and dtype) over source rows
- *          converted to channel-planar FP32 in shared memory.
+ *          owns consecutive output pixels, the even outputs are copies, the
+ *          odd ones the midpoint weights;
+ *          other ratios and dtypes: a thread owns P pixels 32 apart (P = 2 to
+ *          8 by channels and dtype) over source rows converted to
+ *          channel-planar FP32 in shared memory.
  *          waves = blocks per resident block slot (sets the band height).
  * STREAM = one block per (column strip, band of rows), walking down the band
  *          in chunks; every source row is staged and horizontally
@@ -110,8 +113,8 @@ typedef enum { RS_COORD_ASYMMETRIC = 0, RS_COORD_HALF_PIXEL = 1, RS_COORD_ALIGN_
  *          16-byte units (pointer, pitch and W*C multiples of 4 elements):
  *          the register window in its transposed roles (the backward's fused
  *          kernel with the taps of Eqs. 1-5 computed in the kernel). Each
- *          thread owns 2 output elements (strided by 256) of a 512-element
- *          strip for a band of output rows; the source rows the band's taps
+ *          thread owns 2 output elements of a strip of up to 512 elements
+ *          for a band of output rows; the source rows the band's taps
  *          reach are copied with 16-byte cp.async into a three-slot ring and
  *          horizontally interpolated at the thread's columns into a register
  *          window; every output row whose first tap is the window's first
@@ -141,8 +144,8 @@ typedef enum { RS_IMPL_AUTO = 0, RS_IMPL_TILED = 1, RS_IMPL_PLAIN = 2, RS_IMPL_S
  *   (impl RS_IMPL_WINDOW selects it and refuses more taps); beyond that, on
  *   vertical downscales (output rows <= source rows), a vertical-first
  *   streaming kernel (each tile's source rows copied once through a
- *   shared-memory ring, the vertical sums kept in registers, the finished
- *   rows blended horizontally; impl RS_IMPL_STREAM selects it, and refuses
+ *   shared-memory ring, the vertical sums kept in registers, four finished
+ *   rows at a time blended horizontally; impl RS_IMPL_STREAM selects it, and refuses
  *   vertical upscales), else, or with impl RS_IMPL_TILED, a tiled kernel
  *   that holds any number of taps (tiles of 32 output columns: the tile's
  *   footprint rows are interpolated horizontally into shared memory, then
@@ -251,7 +254,8 @@ rs_status rs_resize_normalize(const void* src, const rs_layout* in, void* dst, c
  * planes, at most ~256 MB); it is written by the call and may be reused after
  * the call's work on `stream` has finished. Kernels (opt->impl):
  *   RS_IMPL_AUTO   - WINDOW where it applies, else STREAM, else TILED;
- *   RS_IMPL_WINDOW - one fused pass: each thread keeps the x-transposed
+ *   RS_IMPL_WINDOW - one fused pass (for exact x2 of one channel without
+ *                    the table pass): each thread keeps the x-transposed
  *                    dY rows its y taps need in registers (at most 8
  *                    transposed taps per axis, dY rows of whole aligned
  *                    16-byte units; RS_ERR_INVALID_ARG otherwise); same
@@ -290,8 +294,9 @@ typedef struct {
 /*
  * Batch options (rs_options): coord and cubic_a apply to every image.
  * impl = RS_IMPL_AUTO: bilinear / bicubic images whose source footprint
- *   fits run as register-window items (bands of 256 output rows, source
- *   rows staged 8 at a time, else 4), the rest as tiles; when
+ *   fits run as register-window items (bands of 32 to 256 output rows, by
+ *   the batch's work; source rows staged 8 at a time, else 4), the rest as
+ *   tiles; when
  *   rs_autotune_batched has tuned this batch (same sizes, methods, pitches,
  *   dtype, count and coord) its shape is used instead. An explicit tile_w /
  *   tile_h / threads tiles every image.
@@ -363,7 +368,8 @@ rs_status rs_batched_plan_create(const rs_image_desc* d, int n, rs_dtype dtype,
                                  rs_batched_plan** plan);
 rs_status rs_batched_plan_launch(rs_batched_plan* plan, void* stream);
 /* Kernel launches one replay makes: one persistent launch per non-empty class
- * (window items by method, channel count and footprint tier; tiles). */
+ * (window items by method, channel count and footprint tier; uint8 window
+ * items read in place by method, channel count and direction; tiles). */
 rs_status rs_batched_plan_kernels(const rs_batched_plan* plan, int32_t* kernels);
 rs_status rs_batched_plan_destroy(rs_batched_plan* plan);
 

@@ -879,6 +879,9 @@ k_adj_x2(const Geom g, const float* __restrict__ dY, float* __restrict__ dX, int
     asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
 
+// Exact x2 runs k_adj_x2 wherever its 16-byte copies are aligned. 32 x 3 planes
+// of 512^2 -> 1024^2, k_adj_window -> k_adj_x2: bicubic 125 us and a 4 us table
+// pass -> 86 us, bilinear 94 -> 84 us (503 MB: 75 us at the copy rate).
 static bool adj_x2_ok(const Geom& g, int method, int aa, const void* dY)
 {
     return g.C == 1 && !aa && (method == M_BILINEAR || method == M_BICUBIC) &&

@@ -3,18 +3,19 @@
 // work list in device memory.
 //
 // The host sorts the images into classes. A bilinear / bicubic image whose
-// footprint fits becomes (strip of 1024 output elements, band of output
-// rows) items of the register-window kernel, in the class of its (method,
-// channel count); any other image (nearest, or too large a footprint)
+// footprint fits becomes (strip of output pixels, band of output rows) items
+// of the register-window kernel (uint8 images of up to two source pixels per
+// output pixel: of the form that reads them in place), in the class of its
+// (method, channel count); any other image (nearest, or too large a footprint)
 // becomes output tiles of the tiled kernel, in one class of its own. Each
 // class is a contiguous run of image descriptors with an exclusive prefix
 // sum of their item counts; descriptors and prefixes go to device memory
 // (the caller's workspace, or the library's fixed array for the
 // no-allocation entry point). Each non-empty class is ONE persistent launch,
 // fully specialised for its class: one block per resident slot (SM count x
-// blocks per SM); block b takes items b, b + gridDim.x, ..., finds each
-// item's image by binary search in the class prefix and runs the image's
-// per-block work. No block waits on another. The replayable plan records the
+// blocks per SM); the blocks draw items from the class's counter, find each
+// item's image by binary search in the class prefix and run the image's
+// per-block work. A direct call's launches overlap. The replayable plan records the
 // class launches as independent nodes of one CUDA graph. With
 // RS_FLAG_ANTIALIAS every image is resampled with the antialias taps: window
 // items up to 8 taps per axis, many-tap tiles beyond.
