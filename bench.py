@@ -415,7 +415,7 @@ def run_ours(args, rank, world, local):
                    "out_bytes_per_step": b.out_bytes},
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
                      "frac": achieved / hbm_peak, "traffic": traffic,
-                     "kernel": f"the batch plan ({kernels} k_batched_window / k_batched class launches, one graph)",
+                     "kernel": f"the batch plan ({kernels} k_batched_raw / k_batched_window / k_batched class launches, one graph)",
                      "algorithmic_bytes_per_launch": alg_bytes, "peak_kind": f"{peak_kind} copy bandwidth"},
         "clocks": clk,
         "e2e": e2e,
