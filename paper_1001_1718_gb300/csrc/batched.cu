@@ -99,18 +99,22 @@ struct ItemQueue {
     {
         if (threadIdx.x == 0 && t < total) drawn = atomicAdd(next, 1ull);
     }
-    // every thread of the block, done with the item's shared memory
-    __device__ __forceinline__ void advance()
+    // every thread of the block, done with the item. The drawn number passes
+    // through the start of the dynamic shared memory, between items: an item
+    // may take all that a block can have, which leaves no room for a variable
+    // beside it.
+    __device__ __forceinline__ void advance(float* sm)
     {
-        __shared__ int64_t item;
+        int64_t* const item = reinterpret_cast<int64_t*>(sm);
+        __syncthreads();   // the item's shared memory is free
         if (threadIdx.x == 0) {
             if (drawn + 1 == (unsigned long long)total) *next = 0ull;
-            item = (int64_t)drawn + gridDim.x;
+            *item = (int64_t)drawn + gridDim.x;
         }
         __syncthreads();
-        t = item;
+        t = *item;
         draw();
-        __syncthreads();   // the next item reuses shared memory (and `item`)
+        __syncthreads();   // read by all: the next item may use shared memory
     }
 };
 
@@ -137,7 +141,7 @@ k_batched_window(const BatchImage* __restrict__ imgs, const int64_t* __restrict_
 {
     extern __shared__ __align__(16) float sm[];
     ItemQueue::open();
-    for (ItemQueue q(next, total); q.t < total; q.advance()) {
+    for (ItemQueue q(next, total); q.t < total; q.advance(sm)) {
         const int64_t t = q.t;
         const int k = find_image(start, n, t);
         const BatchImage im = imgs[k];
@@ -175,7 +179,7 @@ k_batched_raw(const BatchImage* __restrict__ imgs, const int64_t* __restrict__ s
 {
     extern __shared__ __align__(16) float sm[];
     ItemQueue::open();
-    for (ItemQueue q(next, total); q.t < total; q.advance()) {
+    for (ItemQueue q(next, total); q.t < total; q.advance(sm)) {
         const int64_t t = q.t;
         const int k = find_image(start, n, t);
         const BatchImage im = imgs[k];
@@ -218,7 +222,7 @@ k_batched_aa_wide(const BatchImage* __restrict__ imgs, const int64_t* __restrict
 {
     extern __shared__ __align__(16) float sm[];
     ItemQueue::open();
-    for (ItemQueue q(next, total); q.t < total; q.advance()) {
+    for (ItemQueue q(next, total); q.t < total; q.advance(sm)) {
         const int64_t t = q.t;
         const int k = find_image(start, n, t);
         const BatchImage im = imgs[k];
@@ -267,7 +271,7 @@ k_batched(const BatchImage* __restrict__ imgs, const int64_t* __restrict__ start
 {
     extern __shared__ __align__(16) float sm[];
     ItemQueue::open();
-    for (ItemQueue q(next, total); q.t < total; q.advance()) {
+    for (ItemQueue q(next, total); q.t < total; q.advance(sm)) {
         const int64_t t = q.t;
         const int k = find_image(start, n, t);
         const BatchImage im = imgs[k];
