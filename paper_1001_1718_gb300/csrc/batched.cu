@@ -59,6 +59,11 @@ static constexpr int kClasses = 33;
 static constexpr int kTileClass = 16;
 static constexpr int kRawClass = 17;
 static constexpr int kRawThreads = kWinThreads;
+// Blocks per SM that the tile kernels' registers leave room for (at most 64 a
+// thread). Without the bound the compiler aimed at more and spilled (40 to 48
+// registers): antialias batches took up to twice as long (one RGBA image of
+// 407 x 114 to 73 x 11, bilinear: 119 us, with the bound 72).
+static constexpr int kTileBlocks = 4;
 static constexpr size_t kWindowSmallSmem = 72 * 1024;
 static constexpr int kHeavyBand = 32;   // band rows of large-footprint and downscaled window items
 
@@ -216,7 +221,7 @@ k_batched_raw(const BatchImage* __restrict__ imgs, const int64_t* __restrict__ s
 
 // Many-tap antialias tiles (kind 2) of any channel count.
 template <typename T>
-__global__ void __launch_bounds__(kAwNT)
+__global__ void __launch_bounds__(kAwNT, kTileBlocks)
 k_batched_aa_wide(const BatchImage* __restrict__ imgs, const int64_t* __restrict__ start, int n, int64_t total,
                   unsigned long long* next, int coord, float a, unsigned int* fault)
 {
@@ -265,7 +270,7 @@ __device__ __forceinline__ void batch_tile_c(const Geom& g, const BatchImage& im
 
 // Tile items of any method and channel count.
 template <typename T>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, kTileBlocks)
 k_batched(const BatchImage* __restrict__ imgs, const int64_t* __restrict__ start, int n, int64_t total,
           unsigned long long* next, int coord, float a, unsigned int* fault)
 {
