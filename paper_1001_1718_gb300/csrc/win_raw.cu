@@ -189,7 +189,7 @@ bool win_raw_default(const Geom& g, int method, int dtype, int nt, int band_cap,
 static int raw_store_mode(const Geom& g, const void* dst, size_t es, int unit, int64_t c_stride)
 {
     const bool ok = g.Wo % kRawP == 0 && reinterpret_cast<uintptr_t>(dst) % unit == 0 && g.dst_pitch * es % unit == 0 &&
-                    (g.planes == 1 || (g.dp.n_stride * es % unit == 0 && g.dp.c_stride * es % unit == 0)) &&
+                    (g.planes == 1 || g.dp.n_stride * es % unit == 0) && (g.dp.cp == 1 || g.dp.c_stride * es % unit == 0) &&
                     c_stride * es % unit == 0;
     return ok ? RAW_WORDS : RAW_ANY;
 }
