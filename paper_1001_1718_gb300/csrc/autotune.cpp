@@ -161,14 +161,21 @@ static bool default_choice(const Geom& g, int method, int dtype, const void* src
     }
     if ((g.Ho >= g.H || dtype == DT_U8) && out_elems >= (int64_t)1 << 22) {
         // Large float outputs of the exact-x2 form (bound by HBM) in five blocks
-        // per slot: their stores start and end evenly (bicubic, two / five:
-        // FP32 4096^2 -> 8192^2 61.6 / 54.2 us, FP16 8192^2 -> 16384^2 116 /
-        // 110); below ~192 MB of output the extra prologues cost more
-        // (BF16 4096^2, 128 MB: 33.3 / 37.3).
-        const bool big_x2 = dtype != DT_U8 && win_is_x2(g) && out_elems * (int64_t)dtype_size(dtype) >= (int64_t)192 << 20;
+        // per slot, four below 320 MB: their stores start and end evenly
+        // (bicubic, two / five: FP32 4096^2 -> 8192^2 61.6 / 54.2 us, FP16
+        // 8192^2 -> 16384^2 116 / 110; bilinear FP32, 32 planes of 249 x 2773 ->
+        // 498 x 5546 84.0 / 72.9; two / four / five, 32 FP16 planes to 3492 x
+        // 910, 203 MB: 70.1 / 70.9 / 72.7); below ~192 MB of output the extra
+        // prologues cost more (BF16 4096^2, 128 MB: 33.3 / 37.3).
+        const int64_t out_bytes = out_elems * (int64_t)dtype_size(dtype);
+        const bool x2 = win_is_x2(g);
+        const int waves = g.Ho < g.H && g.planes == 1 ? 1 : dtype == DT_U8 || !x2 || out_bytes < (int64_t)192 << 20 ? 2
+                        : out_bytes < (int64_t)320 << 20 ? 4 : 5;
         for (int ch : {8, 4}) {
-            const Tuned t{RS_IMPL_WINDOW, 1024, ch, 128, g.Ho < g.H && g.planes == 1 ? 1 : big_x2 ? 5 : 2};
-            if (make_choice(g, method, dtype, src, t, k) && k.window.smem <= (ch == 8 ? 56 : 100) * 1024) return true;
+            const Tuned t{RS_IMPL_WINDOW, 1024, ch, 128, waves};
+            if (!make_choice(g, method, dtype, src, t, k) || k.window.smem > (ch == 8 ? 56 : 100) * 1024) continue;
+            if (k.window.pat) k.window.waves = std::min(waves, win_raw_waves(out_bytes));
+            return true;
         }
     }
     StreamCfg sc = stream_default(g, method, dtype, src);

@@ -138,6 +138,14 @@ int win_raw_block(const Geom& g, int warp_px)
     return (int64_t)g.W > 2 * (int64_t)g.Wo ? std::min(nt, 64) : nt;
 }
 
+// Two blocks per resident slot; one for outputs of at most 32 MB, whose bands
+// would be hardly longer than the rows and copies a block starts with (exact
+// x2, RGB 653 x 1148 bilinear, 9 MB: 5.7 us in one, 7.6 in two, and 6.6 on the
+// form on FP32 windows that this one replaced; grey 32 x 485 x 171 -> 1570 x
+// 553 bilinear, 28 MB: 26.0, 29.2 and 27.4). The two cross near 45 MB (exact
+// x2, 16 planes of 356 x 2900, 66 MB: 28.6 in one, 25.5 in two).
+int win_raw_waves(int64_t out_bytes) { return out_bytes <= (int64_t)32 << 20 ? 1 : 2; }
+
 bool win_raw_config(const Geom& g, int method, int dtype, int nt, int band_cap, WinCfg& c, bool allow_x2)
 {
     c.pat = 0;
@@ -204,7 +212,8 @@ static cudaError_t launch_raw(const Geom& g, void* func, int strip, const void* 
     const int64_t strips = ((int64_t)g.Wo + strip - 1) / strip;
     if (c.band_h <= 0) {
         const int64_t resident = (int64_t)num_sms() * std::max(1, per_sm);
-        const int waves = c.waves > 0 ? c.waves : 2;
+        const int64_t elems = (int64_t)g.Ho * g.Wo * g.C * g.planes;
+        const int waves = c.waves > 0 ? c.waves : win_raw_waves(elems * (int64_t)(no ? dtype_size(no->dtype) : 1));
         // at most `waves` blocks per resident slot: a partial extra wave would run alone
         const int64_t bands = std::max<int64_t>(1, resident * waves / (strips * g.planes));
         c.band_h = (int)std::min<int64_t>(c.band_cap, std::max<int64_t>(1, (g.Ho + bands - 1) / bands));
