@@ -247,7 +247,7 @@ rs_status rs_resize_normalize(const void* src, const rs_layout* in, void* dst, c
     WinCfg raw = c;
     raw.chunk = o.tile_h;
     if ((g.C == 1 || g.C == 3) && win_raw_default(g, method, DT_U8, win_raw_block(g, 128), 256, raw) &&
-        win_raw_norm_ok(g, dst, raw, no))
+        win_raw_norm_ok(g, dst, raw, no, c))
         return cuda_status(launch_win_raw_norm(g, method, src, dst, raw, no, static_cast<cudaStream_t>(stream)));
     return cuda_status(launch_win_norm(g, method, out_dtype, src, dst, c, no, static_cast<cudaStream_t>(stream)));
 }

@@ -215,8 +215,9 @@ int win_raw_threads(int Wo, int warp_px);
 int win_raw_block(const Geom& g, int warp_px);   // its threads per block for a problem
 int win_raw_waves(int64_t out_bytes);           // its default blocks per resident slot
 cudaError_t launch_win_raw(const Geom& g, int method, const void* src, void* dst, WinCfg c, cudaStream_t st);
-// Whether the pre-process's output rows suit the form (win_raw.cu).
-bool win_raw_norm_ok(const Geom& g, const void* dst, const WinCfg& c, const NormOut& no);
+// Whether the pre-process's output suits the form better than the FP32 form of
+// configuration fp32 (win_raw.cu).
+bool win_raw_norm_ok(const Geom& g, const void* dst, const WinCfg& c, const NormOut& no, const WinCfg& fp32);
 cudaError_t launch_win_raw_norm(const Geom& g, int method, const void* src, void* dst, WinCfg c, const NormOut& no,
                                 cudaStream_t st);
 cudaError_t launch_win(const Geom& g, int method, int dtype, const void* src, void* dst, WinCfg c, cudaStream_t st);

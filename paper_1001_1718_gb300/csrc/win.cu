@@ -117,8 +117,10 @@ bool win_config(const Geom& g, int method, int dtype, WinCfg& c, bool allow_x2)
     const int P = win_pixels(g.C, dtype, x2);
     // narrow rows: only the warps they fill (the batch's blocks are all alike;
     // a downscale's block spends most of its time staging rows, which idle
-    // lanes share)
-    c.nt = allow_x2 && g.Wo >= g.W ? win_raw_threads(g.Wo, 32 * P) : kWinThreads;
+    // lanes share, and so does each of a few short rows' blocks: RGBA
+    // pre-process of 29 x 67 doubled 3.4 us, in narrow blocks 3.9)
+    const bool narrow = allow_x2 && g.Wo >= g.W && (int64_t)g.Ho * g.planes > 2 * num_sms();
+    c.nt = narrow ? win_raw_threads(g.Wo, 32 * P) : kWinThreads;
     const int SP = c.nt * P;
     c.pat = 0;
     // source pixels a strip's footprint can span

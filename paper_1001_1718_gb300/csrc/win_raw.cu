@@ -239,11 +239,20 @@ cudaError_t launch_win_raw(const Geom& g, int method, const void* src, void* dst
     return launch_raw(g, func, raw_strip(c.nt, raw_overlap(mode, 1)), src, dst, c, nullptr, st);
 }
 
-bool win_raw_norm_ok(const Geom& g, const void* dst, const WinCfg& c, const NormOut& no)
+bool win_raw_norm_ok(const Geom& g, const void* dst, const WinCfg& c, const NormOut& no, const WinCfg& fp32)
 {
+    const bool x2 = c.pat == kRawX2 + 1;
     // three FP32 planes of an exact x2 are all stores: the form on consecutive
     // pairs keeps them a little faster (16 x 512^2 bicubic 38 us, here 39.5)
-    if (c.pat == kRawX2 + 1 && no.dtype == DT_F32 && g.C == 3) return false;
+    if (x2 && no.dtype == DT_F32 && g.C == 3) return false;
+    // Small outputs, whose shortest bands (one row; two of an exact x2) all run
+    // at once on the FP32 forms: a block is all start-up, which takes longer
+    // here (RGB 54 x 55 -> 27 x 28 bicubic 7.3 us, on FP32 rows 3.9; RGB exact
+    // x2 to 152 x 340 bilinear 3.7 and 2.9).
+    const int px = fp32.nt * win_pixels(g.C, DT_U8, x2);
+    const int64_t blocks = ((int64_t)g.Wo + px - 1) / px * ((g.Ho + x2) / (x2 ? 2 : 1)) * g.planes;
+    const int64_t per_sm = std::min<int64_t>(x2 ? 4 : 2, 228 * 1024 / ((int64_t)fp32.smem + 1024));
+    if (blocks <= num_sms() * per_sm) return false;
     const size_t es = dtype_size(no.dtype);
     return c.pat == 2 + 1 || c.pat == 4 + 1 || raw_store_mode(g, dst, es, kRawP * (int)es, no.c_stride) == RAW_WORDS;
 }

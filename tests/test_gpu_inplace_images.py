@@ -1,5 +1,6 @@
 """The uint8 in-place form on several images at once: interleaved stacks whose
-images start on a store's boundary and off it."""
+images start on a store's boundary and off it, and the pre-process on enough
+images that the form is taken (a few short rows stay on the FP32 forms)."""
 import numpy as np
 import pytest
 import torch
@@ -25,4 +26,24 @@ def test_interleaved_stacks(W, Wo, C, method):
         assert torch.equal(y, ref), (gap, off)
         y.fill_(77)
         assert (buf == 77).all(), (gap, off)   # nothing written between the images
+    assert rs.debug_fault() == 0
+
+
+@pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("W,Wo", [(100, 256), (300, 512), (455, 455), (455, 456), (700, 455), (1024, 512), (9, 5),
+                                  (130, 260), (650, 250), (515, 255)])
+def test_normalize_stacks(W, Wo, dtype):
+    mean, std = (123.675, 116.28, 103.53), (58.395, 57.12, 57.375)
+    N = 48
+    for C in (1, 3):
+        for method, coord in (("bilinear", "half_pixel"), ("bicubic", "asymmetric")):
+            Ho = 82 if Wo == 2 * W else 29
+            g = np.random.default_rng(W)
+            x = torch.from_numpy(g.integers(0, 256, (N, 41, W, C), dtype=np.uint8)).cuda()
+            y = rs.resize_normalize(x, (Ho, Wo), method, mean[:C], std[:C], dtype=dtype, coord=coord)
+            v = rs.resize(x.float(), (Ho, Wo), method, coord=coord, impl="tiled").double().permute(0, 3, 1, 2)
+            sc = torch.tensor([np.float32(1) / np.float32(s) for s in std[:C]], device="cuda").double().view(1, C, 1, 1)
+            bi = torch.tensor([-np.float32(m) / np.float32(s) for m, s in zip(mean, std)][:C], device="cuda").double()
+            # one FP32 multiply-add of the FP32 value, then one rounding to the output type
+            assert torch.equal(y, (v * sc + bi.view(1, C, 1, 1)).float().to(dtype))
     assert rs.debug_fault() == 0
