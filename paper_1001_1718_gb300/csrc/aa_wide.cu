@@ -20,8 +20,11 @@
 
 namespace rs {
 
+// (four blocks per SM: shared memory rarely lets more in, and without the bound
+// the compiler kept to 32 registers a thread: FP32 RGBA 894 x 2591 -> 7 x 22
+// bilinear 1540 us, with it 1307)
 template <int C, typename T, typename TO, bool NORM>
-__global__ void __launch_bounds__(kAwNT)
+__global__ void __launch_bounds__(kAwNT, 4)
 k_aa_wide(const Geom g, const T* __restrict__ src, TO* __restrict__ dst, const AaWideCfg cfg, const NormOut no,
           unsigned int* fault)
 {
