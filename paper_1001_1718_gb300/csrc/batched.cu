@@ -327,10 +327,13 @@ static bool image_tile(const Geom& g, int method, int tile_w, int h_cap, int thr
 
 // Shape of a batch's items: every image as tiles, or bilinear / bicubic
 // images as register-window items of `band` output rows whose source rows
-// are staged `chunk` at a time (chunk 0: 8, else 4 when 8 does not fit).
+// are staged `chunk` at a time (chunk 0: 8, else 4 when 8 does not fit);
+// inplace: uint8 images of up to two source pixels per output pixel are read
+// in place.
 struct BatchShape {
     bool tiled;
     int chunk, band;
+    bool inplace = true;
 };
 
 // Antialias taps (RS_FLAG_ANTIALIAS): window items with at most K = 4 or 8
@@ -382,11 +385,13 @@ static rs_status prepare_image_aa(const rs_image_desc& x, const Geom& g, int dty
 
 // Validates one descriptor and fills its device descriptor: window items
 // (bilinear / bicubic, footprint within ~100 KB of shared memory) or tiles.
-// Returns the class, item count and shared-memory need.
+// Returns the class, the window class of an image read in place (general;
+// else -1), item count and shared-memory need.
 static rs_status prepare_image(const rs_image_desc& x, int dtype, const rs_options& o, const BatchShape& sh,
-                               int tile_w, int h_cap, int threads, BatchImage& im, int& cls, int64_t& items,
-                               size_t& smem)
+                               int tile_w, int h_cap, int threads, BatchImage& im, int& cls, int& general,
+                               int64_t& items, size_t& smem)
 {
+    general = -1;
     const int64_t es = (int64_t)dtype_size(dtype);
     if (!x.src || !x.dst) return RS_ERR_INVALID_ARG;
     if (!dim_ok(x.H) || !dim_ok(x.W) || !dim_ok(x.Ho) || !dim_ok(x.Wo)) return RS_ERR_INVALID_ARG;
@@ -420,7 +425,8 @@ static rs_status prepare_image(const rs_image_desc& x, int dtype, const rs_optio
             raw.chunk = sh.chunk;
             // a downscale's output row takes several source rows: shorter bands
             const int band = x.Ho < x.H ? std::max(std::min(sh.band, kHeavyBand), (int)((int64_t)sh.band * x.Ho / x.H)) : sh.band;
-            if (win_raw_default(g, x.method, dtype, kRawThreads, band, raw, false) && raw.pat <= 3) {   // uint8 read in place, up to 2 source pixels per output pixel
+            const int window_cls = (wc.smem <= kWindowSmallSmem ? 0 : 8) + (x.method == RS_BILINEAR ? 0 : 4) + (x.C - 1);
+            if (sh.inplace && win_raw_default(g, x.method, dtype, kRawThreads, band, raw, false) && raw.pat <= 3) {   // uint8 read in place, up to 2 source pixels per output pixel
                 im.kind = 3;
                 im.pat = raw.pat;
                 im.chunk = raw.chunk;
@@ -435,6 +441,7 @@ static rs_status prepare_image(const rs_image_desc& x, int dtype, const rs_optio
                 items = (int64_t)im.tiles_x * ((x.Ho + im.band_h - 1) / im.band_h);
                 smem = raw.smem;
                 cls = kRawClass + (raw.pat == 3 ? 8 : 0) + (x.method == RS_BILINEAR ? 0 : 4) + (x.C - 1);
+                general = window_cls;
                 return RS_OK;
             }
             im.kind = 1;
@@ -454,7 +461,7 @@ static rs_status prepare_image(const rs_image_desc& x, int dtype, const rs_optio
             im.tiles_x = (int)(((int64_t)x.Wo + sp - 1) / sp);
             items = (int64_t)im.tiles_x * ((x.Ho + im.band_h - 1) / im.band_h);
             smem = wc.smem;
-            cls = (wc.smem <= kWindowSmallSmem ? 0 : 8) + (x.method == RS_BILINEAR ? 0 : 4) + (x.C - 1);
+            cls = window_cls;
             return RS_OK;
         }
     }
@@ -580,14 +587,29 @@ static rs_status batch_layout(const rs_image_desc* d, int n, int dtype, const rs
     L.threads = o.threads ? o.threads : 256;
     if (L.threads != 128 && L.threads != 256) return RS_ERR_INVALID_ARG;
     L.n = n;
-    for (int c = 0; c < kClasses; ++c) { L.count[c] = 0; L.total[c] = 0; L.smem[c] = 0; }
     const int64_t es = (int64_t)dtype_size(dtype);
-    for (int k = 0; k < n; ++k) {
-        size_t sm = 0;
-        s = prepare_image(d[k], dtype, o, sh, tile_w, h_cap, L.threads, tmp_imgs[k], tmp_cls[k], tmp_items[k], sm);
-        if (s != RS_OK) return s;
-        L.count[tmp_cls[k]]++;
-        L.smem[tmp_cls[k]] = std::max(L.smem[tmp_cls[k]], sm);
+    // Reading in place splits the window classes (by direction, and from the
+    // images beyond its ratios). Each launch more costs a few microseconds:
+    // batches of all channel counts, which it would give six launches or more,
+    // need about 200 items for each to pay (110 images of 1 to 4 channels and
+    // some 90 pixels a side: 26 launches 106 us, 15 on FP32 rows 59).
+    for (sh.inplace = true;; sh.inplace = false) {
+        bool general[kClasses] = {};   // the classes if none is read in place
+        int64_t inplace = 0;           // items read in place
+        int more = 0;
+        for (int c = 0; c < kClasses; ++c) { L.count[c] = 0; L.total[c] = 0; L.smem[c] = 0; }
+        for (int k = 0; k < n; ++k) {
+            size_t sm = 0;
+            int gen = -1;
+            s = prepare_image(d[k], dtype, o, sh, tile_w, h_cap, L.threads, tmp_imgs[k], tmp_cls[k], gen, tmp_items[k], sm);
+            if (s != RS_OK) return s;
+            L.count[tmp_cls[k]]++;
+            L.smem[tmp_cls[k]] = std::max(L.smem[tmp_cls[k]], sm);
+            general[gen >= 0 ? gen : tmp_cls[k]] = true;
+            if (gen >= 0) inplace += tmp_items[k];
+        }
+        for (int c = 0; c < kClasses; ++c) more += (L.count[c] > 0) - general[c];
+        if (inplace == 0 || more < 6 || inplace >= 200 * (int64_t)more) break;
     }
     // No destination may overlap any source or another destination.
     auto src_bytes = [&](const rs_image_desc& x) { return ((int64_t)(x.H - 1) * x.src_pitch + (int64_t)x.W * x.C) * es; };
