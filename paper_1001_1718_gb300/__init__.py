@@ -151,8 +151,17 @@ def _remember(key, call) -> None:
 
 
 def _dense_layout(shape, layout: str) -> B.RsLayout:
-    """rs_layout of a new contiguous tensor of `shape`."""
-    return _layout(torch.empty(shape, dtype=torch.uint8, device="meta"), layout)
+    """rs_layout of a new contiguous tensor of `shape` (as _layout gives it)."""
+    n = len(shape)
+    if not 2 <= n <= 4:
+        raise ValueError(f"{layout} layout wants a 2-, 3- or 4-D tensor")
+    N = shape[0] if n == 4 else 1
+    if layout == "hwc":
+        H, W, C = (*shape, 1) if n == 2 else shape[-3:]
+        return B.RsLayout(N, C, H, W, H * W * C, 1, W * C, C)
+    H, W = shape[-2:]
+    C = 1 if n == 2 else shape[-3]
+    return B.RsLayout(N, C, H, W, C * H * W, H * W, W, 1)
 
 
 def _opts(coord, cubic_a, impl, tile, threads, waves=0, antialias=False) -> B.RsOptions:
@@ -162,6 +171,25 @@ def _opts(coord, cubic_a, impl, tile, threads, waves=0, antialias=False) -> B.Rs
     if antialias:
         o.flags = B.RS_FLAG_ANTIALIAS
     return o
+
+
+def _options(opts):
+    """The marshalled rs_options of (coord, a, impl, tile, threads, waves,
+    antialias): calls on new sizes mostly come with the same ones."""
+    o = _CALLS.get(opts)
+    if o is None:
+        o = ctypes.byref(_opts(*opts))
+        _remember(opts, o)
+    return o
+
+
+def _floats(values: tuple):
+    """A host float array of the values."""
+    f = _CALLS.get(values)
+    if f is None:
+        f = (ctypes.c_float * len(values))(*values)
+        _remember(values, f)
+    return f
 
 
 def resize(x: torch.Tensor, size: Sequence[int], method="bilinear", *, layout: str = "hwc",
@@ -183,15 +211,16 @@ def resize(x: torch.Tensor, size: Sequence[int], method="bilinear", *, layout: s
         _require_cuda(out)
         if out.dtype != x.dtype:
             raise ValueError("out must have the dtype of x")
-    key = ("resize", x.shape, x.stride(), x.dtype, Ho, Wo, _code(METHODS, method, "method"), layout,
-           _code(COORDS, coord, "coord"), a, _code(IMPLS, impl, "impl"), tile, threads, waves, antialias,
+    m = _code(METHODS, method, "method")
+    opts = (_code(COORDS, coord, "coord"), a, _code(IMPLS, impl, "impl"), tile, threads, waves, antialias)
+    key = ("resize", x.shape, x.stride(), x.dtype, Ho, Wo, m, layout, opts,
            out is not None and (out.shape, out.stride()))
     call = _CALLS.get(key)
     if call is None:
+        Li = _layout(x, layout)
         shape = _out_shape(x, layout, Ho, Wo)
         Lo = _dense_layout(shape, layout) if out is None else _layout(out, layout)
-        call = (shape, ctypes.byref(_layout(x, layout)), ctypes.byref(Lo), _dtype(x),
-                _code(METHODS, method, "method"), ctypes.byref(_opts(coord, a, impl, tile, threads, waves, antialias)))
+        call = (shape, ctypes.byref(Li), ctypes.byref(Lo), _dtype(x), m, _options(opts))
         _remember(key, call)
     shape, Li, Lo, dt, m, o = call
     if out is None:
@@ -222,9 +251,10 @@ def resize_normalize(x: torch.Tensor, size: Sequence[int], method="bilinear", me
         raise ValueError(f"unsupported output dtype {dtype}") from None
     Ho, Wo = int(size[0]), int(size[1])
     a, chunk, antialias = float(cubic_a), int(chunk), bool(antialias)
-    mean, std = tuple(float(v) for v in mean), tuple(float(v) for v in std)
-    key = ("normalize", x.shape, x.stride(), odt, Ho, Wo, _code(METHODS, method, "method"), mean, std,
-           _code(COORDS, coord, "coord"), a, _code(IMPLS, impl, "impl"), chunk, antialias,
+    mean, std = tuple(map(float, mean)), tuple(map(float, std))
+    m = _code(METHODS, method, "method")
+    opts = (_code(COORDS, coord, "coord"), a, _code(IMPLS, impl, "impl"), (0, chunk), 0, 0, antialias)
+    key = ("normalize", x.shape, x.stride(), odt, Ho, Wo, m, mean, std, opts,
            out is not None and (out.shape, out.stride(), out.dtype))
     call = _CALLS.get(key)
     if call is None:
@@ -240,9 +270,7 @@ def resize_normalize(x: torch.Tensor, size: Sequence[int], method="bilinear", me
         Li = _layout(x, "hwc")
         if len(mean) != C or len(std) != C:
             raise ValueError("mean and std need one value per channel")
-        call = (shape, ctypes.byref(Li), ctypes.byref(Lo), _code(METHODS, method, "method"),
-                (ctypes.c_float * C)(*mean), (ctypes.c_float * C)(*std),
-                ctypes.byref(_opts(coord, a, impl, (0, chunk), 0, 0, antialias)))
+        call = (shape, ctypes.byref(Li), ctypes.byref(Lo), m, _floats(mean), _floats(std), _options(opts))
         _remember(key, call)
     shape, Li, Lo, m, cm, cs, o = call
     if out is None:
@@ -276,16 +304,16 @@ def resize_backward(grad_out: torch.Tensor, in_hw, method="bilinear", *, layout:
     _require_cuda(grad_out)
     H, W = int(in_hw[0]), int(in_hw[1])
     a, antialias = float(cubic_a), bool(antialias)
-    key = ("backward", grad_out.shape, grad_out.stride(), grad_out.dtype, H, W, _code(METHODS, method, "method"),
-           layout, _code(COORDS, coord, "coord"), a, _code(IMPLS, impl, "impl"), antialias,
+    m = _code(METHODS, method, "method")
+    opts = (_code(COORDS, coord, "coord"), a, _code(IMPLS, impl, "impl"), (0, 0), 0, 0, antialias)
+    key = ("backward", grad_out.shape, grad_out.stride(), grad_out.dtype, H, W, m, layout, opts,
            grad_in is not None and (grad_in.shape, grad_in.stride()))
     call = _CALLS.get(key)
     if call is None:
         shape = _out_shape(grad_out, layout, H, W)
         Lo = ctypes.byref(_layout(grad_out, layout))
         Li = ctypes.byref(_dense_layout(shape, layout) if grad_in is None else _layout(grad_in, layout))
-        o = ctypes.byref(_opts(coord, a, impl, None, 0, 0, antialias))
-        m = _code(METHODS, method, "method")
+        o = _options(opts)
         n = ctypes.c_size_t(0)
         B.check(lib().rs_resize_backward_workspace(Lo, Li, m, o, ctypes.byref(n)), "rs_resize_backward_workspace")
         call = (shape, Lo, Li, _dtype(grad_out), m, o, n.value)

@@ -592,7 +592,7 @@ static rs_status batch_layout(const rs_image_desc* d, int n, int dtype, const rs
     // images beyond its ratios). Each launch more costs a few microseconds:
     // batches of all channel counts, which it would give six launches or more,
     // need about 200 items for each to pay (110 images of 1 to 4 channels and
-    // some 90 pixels a side: 26 launches 106 us, 15 on FP32 rows 59).
+    // some 90 pixels a side: 26 launches 106 us, 15 on FP32 rows 52).
     for (sh.inplace = true;; sh.inplace = false) {
         bool general[kClasses] = {};   // the classes if none is read in place
         int64_t inplace = 0;           // items read in place
