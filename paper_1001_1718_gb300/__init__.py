@@ -173,22 +173,22 @@ def _opts(coord, cubic_a, impl, tile, threads, waves=0, antialias=False) -> B.Rs
     return o
 
 
-def _options(opts):
+def _options(opts, key):
     """The marshalled rs_options of (coord, a, impl, tile, threads, waves,
     antialias): calls on new sizes mostly come with the same ones."""
-    o = _CALLS.get(opts)
+    o = _CALLS.get(key)
     if o is None:
         o = ctypes.byref(_opts(*opts))
-        _remember(opts, o)
+        _remember(key, o)
     return o
 
 
-def _floats(values: tuple):
+def _floats(values: tuple, key):
     """A host float array of the values."""
-    f = _CALLS.get(values)
+    f = _CALLS.get(key)
     if f is None:
         f = (ctypes.c_float * len(values))(*values)
-        _remember(values, f)
+        _remember(key, f)
     return f
 
 
@@ -213,14 +213,15 @@ def resize(x: torch.Tensor, size: Sequence[int], method="bilinear", *, layout: s
             raise ValueError("out must have the dtype of x")
     m = _code(METHODS, method, "method")
     opts = (_code(COORDS, coord, "coord"), a, _code(IMPLS, impl, "impl"), tile, threads, waves, antialias)
-    key = ("resize", x.shape, x.stride(), x.dtype, Ho, Wo, m, layout, opts,
+    okey = opts if a else (opts, repr(a))   # 0.0 == -0.0, but they are other arguments
+    key = ("resize", x.shape, x.stride(), x.dtype, Ho, Wo, m, layout, okey,
            out is not None and (out.shape, out.stride()))
     call = _CALLS.get(key)
     if call is None:
         Li = _layout(x, layout)
         shape = _out_shape(x, layout, Ho, Wo)
         Lo = _dense_layout(shape, layout) if out is None else _layout(out, layout)
-        call = (shape, ctypes.byref(Li), ctypes.byref(Lo), _dtype(x), m, _options(opts))
+        call = (shape, ctypes.byref(Li), ctypes.byref(Lo), _dtype(x), m, _options(opts, okey))
         _remember(key, call)
     shape, Li, Lo, dt, m, o = call
     if out is None:
@@ -254,7 +255,9 @@ def resize_normalize(x: torch.Tensor, size: Sequence[int], method="bilinear", me
     mean, std = tuple(map(float, mean)), tuple(map(float, std))
     m = _code(METHODS, method, "method")
     opts = (_code(COORDS, coord, "coord"), a, _code(IMPLS, impl, "impl"), (0, chunk), 0, 0, antialias)
-    key = ("normalize", x.shape, x.stride(), odt, Ho, Wo, m, mean, std, opts,
+    okey = opts if a else (opts, repr(a))
+    mkey = mean if 0.0 not in mean else repr(mean)
+    key = ("normalize", x.shape, x.stride(), odt, Ho, Wo, m, mkey, std, okey,
            out is not None and (out.shape, out.stride(), out.dtype))
     call = _CALLS.get(key)
     if call is None:
@@ -270,7 +273,8 @@ def resize_normalize(x: torch.Tensor, size: Sequence[int], method="bilinear", me
         Li = _layout(x, "hwc")
         if len(mean) != C or len(std) != C:
             raise ValueError("mean and std need one value per channel")
-        call = (shape, ctypes.byref(Li), ctypes.byref(Lo), m, _floats(mean), _floats(std), _options(opts))
+        call = (shape, ctypes.byref(Li), ctypes.byref(Lo), m, _floats(mean, mkey), _floats(std, std),
+                _options(opts, okey))
         _remember(key, call)
     shape, Li, Lo, m, cm, cs, o = call
     if out is None:
@@ -306,14 +310,15 @@ def resize_backward(grad_out: torch.Tensor, in_hw, method="bilinear", *, layout:
     a, antialias = float(cubic_a), bool(antialias)
     m = _code(METHODS, method, "method")
     opts = (_code(COORDS, coord, "coord"), a, _code(IMPLS, impl, "impl"), (0, 0), 0, 0, antialias)
-    key = ("backward", grad_out.shape, grad_out.stride(), grad_out.dtype, H, W, m, layout, opts,
+    okey = opts if a else (opts, repr(a))
+    key = ("backward", grad_out.shape, grad_out.stride(), grad_out.dtype, H, W, m, layout, okey,
            grad_in is not None and (grad_in.shape, grad_in.stride()))
     call = _CALLS.get(key)
     if call is None:
         shape = _out_shape(grad_out, layout, H, W)
         Lo = ctypes.byref(_layout(grad_out, layout))
         Li = ctypes.byref(_dense_layout(shape, layout) if grad_in is None else _layout(grad_in, layout))
-        o = _options(opts)
+        o = _options(opts, okey)
         n = ctypes.c_size_t(0)
         B.check(lib().rs_resize_backward_workspace(Lo, Li, m, o, ctypes.byref(n)), "rs_resize_backward_workspace")
         call = (shape, Lo, Li, _dtype(grad_out), m, o, n.value)
