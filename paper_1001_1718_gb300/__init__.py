@@ -358,7 +358,15 @@ assert _DESC.size == ctypes.sizeof(B.RsImageDesc)
 
 
 def _descs(srcs, dsts, methods) -> tuple:
+    """The descriptors and their number."""
+    return _describe(srcs, dsts, methods)[:2]
+
+
+def _describe(srcs, dsts, methods) -> tuple:
+    """The descriptors, their number, and whether an image's rows shrink more
+    than 16 times."""
     n = len(srcs)
+    shrunk = False
     buf = bytearray(n * _DESC.size)
     codes = [_code(METHODS, methods[k], "method") for k in range(n)]
     at = 0
@@ -371,7 +379,9 @@ def _descs(srcs, dsts, methods) -> tuple:
             raise ValueError("batched images need dense pixels (pitched rows are fine)")
         _DESC.pack_into(buf, at, s.data_ptr(), d.data_ptr(), H, W, C, Ho, Wo, m, sr, dr)
         at += _DESC.size
-    return (B.RsImageDesc * n).from_buffer(buf), n
+        if W > 16 * Wo:
+            shrunk = True
+    return (B.RsImageDesc * n).from_buffer(buf), n, shrunk
 
 
 def batched_workspace_bytes(srcs, dsts, methods) -> int:
@@ -397,12 +407,16 @@ def resize_batched(srcs: Sequence[torch.Tensor], sizes, methods, *, coord="asymm
     if outs is None:
         outs = [torch.empty((int(h), int(w), s.shape[2]), dtype=s.dtype, device=s.device)
                 for s, (h, w) in zip(srcs, sizes)]
-    arr, n = _descs(srcs, outs, methods)
+    arr, n, shrunk = _describe(srcs, outs, methods)
     dt = _dtype(srcs[0])
-    nbytes = _CALLS.get(("batch", n))   # the call itself checks the descriptors again
+    # The query refuses what the call refuses (it checks the descriptors again)
+    # and batches whose default tiles do not fit in shared memory: with rows of
+    # 1/16 and more they always do.
+    nbytes = None if shrunk else _CALLS.get(("batch", n))
     if nbytes is None:
         nbytes = _batch_bytes(arr, n, dt)
-        _remember(("batch", n), nbytes)
+        if not shrunk:
+            _remember(("batch", n), nbytes)
     if workspace is None or workspace.numel() * workspace.element_size() < nbytes:
         workspace = torch.empty(max(1, nbytes), dtype=torch.uint8, device=srcs[0].device)
     o = _opts(coord, cubic_a, impl, tile, threads, 0, antialias)
