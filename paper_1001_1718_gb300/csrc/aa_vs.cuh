@@ -16,7 +16,9 @@
 // output row whose taps can include the row at once (2 bilinear, 4 bicubic:
 // the stretched kernel is NA output steps long, and output row i + NA starts
 // at or below row i's last tap). A per-row table holds the row's weight in
-// each set, row i in set i mod NA, 0 elsewhere. The loop over output rows is
+// each set, row i in set i mod NA, 0 elsewhere, as the pair that a packed FMA
+// takes; where the pairs of a tile's rows do not fit in shared memory the table
+// holds the weights once and the pairs of one chunk at a time (single). The loop over output rows is
 // unrolled four times, so the sets are registers with fixed roles: row i is
 // complete where its taps end. Four complete rows go to shared memory as two
 // interleaved pairs, and between two barriers the block blends them with the
@@ -38,7 +40,8 @@
 
 namespace rs {
 
-static constexpr int kVsNT = 128;  // threads per block, at most
+static constexpr int kVsNT = 128;     // threads per block, at most
+static constexpr int kVsMaxNT = 256;  // where one output column's footprint asks for more
 
 // Footprint elements per thread: 8 bytes or halves, 4 floats.
 constexpr __host__ __device__ int vs_elems(int es) { return es == 4 ? 4 : 8; }
@@ -79,8 +82,9 @@ __device__ __forceinline__ void aa_vs_body(const Geom& g, const T* __restrict__ 
     const int slot_bytes = vs_rows_bytes(R, S);
     unsigned char* RAW = reinterpret_cast<unsigned char*>(sm);                           // [3] slots
     float2* V = reinterpret_cast<float2*>(RAW + (size_t)3 * slot_bytes);                 // [2][ve] row pairs
-    float2* YW = V + 2 * (size_t)cfg.ve;                                                 // [nr][NA] (w, w)
-    float* WX = reinterpret_cast<float*>(YW + (size_t)cfg.nr * NA);                      // [TW][KX]
+    float2* YW = V + 2 * (size_t)cfg.ve;                                                 // [nr][NA] (w, w), or
+    float* YS = reinterpret_cast<float*>(YW + (size_t)(cfg.single ? R : cfg.nr) * NA);   // the current chunk's and [nr][NA] w
+    float* WX = YS + (cfg.single ? (size_t)cfg.nr * NA : 0);                             // [TW][KX]
     int* LX = reinterpret_cast<int*>(WX + (size_t)TW * cfg.KX);                          // [TW] first x tap - px_lo
     int* CX = LX + TW;                                                                   // [TW] x tap counts
     int* YH = CX + TW;                                                                   // [TH] last y tap + 1 - r_lo
@@ -115,7 +119,11 @@ __device__ __forceinline__ void aa_vs_body(const Geom& g, const T* __restrict__ 
     copy_rows(RAW + slot_bytes, R);
 
     // ---- tap tables ----
-    for (int e = tid; e < nr * NA; e += NT) YW[e] = make_float2(0.0f, 0.0f);
+    if (cfg.single)
+        #pragma unroll 1
+        for (int e = tid; e < nr * NA; e += NT) YS[e] = 0.0f;
+    else
+        for (int e = tid; e < nr * NA; e += NT) YW[e] = make_float2(0.0f, 0.0f);
     __syncthreads();
     for (int i = tid; i < ni + nj; i += NT) {
         if (i >= ni) {
@@ -129,17 +137,19 @@ __device__ __forceinline__ void aa_vs_body(const Geom& g, const T* __restrict__ 
         int lo, hi;
         aa_range(i0 + i, g.H, g.Ho, m, lo, hi);
         const float inv2F = 1.0f / (2.0f * (float)max(g.H, g.Ho));
-        float2* col = YW + (size_t)(lo - r_lo) * NA + i % NA;
+        const int step = cfg.single ? NA : 2 * NA;   // floats per row
+        float* col = (cfg.single ? YS : reinterpret_cast<float*>(YW)) + (size_t)(lo - r_lo) * step + i % NA * (step / NA);
         float tot = 0.0f;
         for (int k = 0; k < hi - lo; ++k) {
             const float v = aa_kernel(lo + k, i0 + i, g.H, g.Ho, inv2F, m, g.a);
-            col[(size_t)k * NA].x = v;
+            col[(size_t)k * step] = v;
             tot += v;
         }
         const float inv = tot != 0.0f ? 1.0f / tot : 1.0f;
         for (int k = 0; k < hi - lo; ++k) {
-            const float w = col[(size_t)k * NA].x * inv;
-            col[(size_t)k * NA] = make_float2(w, w);
+            const float w = col[(size_t)k * step] * inv;
+            if (cfg.single) col[(size_t)k * step] = w;
+            else *reinterpret_cast<float2*>(col + (size_t)k * step) = make_float2(w, w);
         }
         YH[i] = hi - r_lo;
     }
@@ -163,6 +173,16 @@ __device__ __forceinline__ void aa_vs_body(const Geom& g, const T* __restrict__ 
     int y = 0, y_end = min(R, nr), cidx = 0;   // next row, end of the current chunk
     int p = (int)(row_at(RAW, 0) - RAW) + eoff;   // the next row's first owned byte in shared memory
     const float2* yw = YW;
+    auto pair_weights = [&]() {   // single: rows y .. y_end - 1 as pairs, between two barriers
+        #pragma unroll 1
+        for (int e = tid; e < (y_end - y) * NA; e += NT) {
+            const float w = YS[y * NA + e];
+            YW[e] = make_float2(w, w);
+        }
+        yw = YW;
+        __syncthreads();
+    };
+    if (cfg.single) pair_weights();
     auto next_chunk = [&]() {
         ++cidx;
         unsigned char* freed = cur;
@@ -172,6 +192,7 @@ __device__ __forceinline__ void aa_vs_body(const Geom& g, const T* __restrict__ 
         copy_rows(freed, (cidx + 2) * R);
         p = (int)(row_at(cur, y) - RAW) + eoff;
         y_end = min(y + R, nr);
+        if (cfg.single) pair_weights();
     };
     // the row at p into every set
     auto add_row = [&]() {

@@ -35,7 +35,7 @@ k_aa_wide(const Geom g, const T* __restrict__ src, TO* __restrict__ dst, const A
 }
 
 template <int C, typename T, typename TO, bool NORM, int NA, bool AL>
-__global__ void __launch_bounds__(kVsNT, 4)
+__global__ void __launch_bounds__(kVsMaxNT, 2)
 k_aa_vs(const Geom g, const T* __restrict__ src, TO* __restrict__ dst, const AaVsCfg cfg, const NormOut no,
         unsigned int* fault)
 {
@@ -114,8 +114,6 @@ bool aa_vs_config(const Geom& g, int method, int dtype, AaVsCfg& c)
     if (g.C < 1 || g.C > 4 || g.Ho > g.H) return false;
     const int es = (int)dtype_size(dtype), E = vs_elems(es);
     c.aligned = g.src_pitch % E == 0;
-    const int slack = c.aligned ? E - 1 : 0;   // owned elements before the footprint
-    const int cap = kVsNT * E - slack;
     c.method = method;
     c.NA = method == M_BILINEAR ? 2 : 4;
     int s8 = aa_span_bound(std::min(8, g.Wo), g.W, g.Wo, method);
@@ -125,6 +123,13 @@ bool aa_vs_config(const Geom& g, int method, int dtype, AaVsCfg& c)
         if (s8 * g.C > 1024) return false;
     }
     c.KX = aa_span_bound(1, g.W, g.Wo, method);
+    int slack = c.aligned ? E - 1 : 0;   // owned elements before the footprint
+    int cap = kVsNT * E - slack;
+    if (c.KX * g.C > cap) {   // one column's footprint is wider: more threads (FP32), no element before it
+        c.aligned = 0;
+        slack = 0;
+        cap = std::min(kVsMaxNT * E, 1024);
+    }
     int tw = 1;
     while (tw < std::min(g.Wo, 1024) && aa_span_bound(tw + 1, g.W, g.Wo, method) * g.C <= cap) ++tw;
     const int tiles = (g.Wo + tw - 1) / tw;
@@ -133,9 +138,8 @@ bool aa_vs_config(const Geom& g, int method, int dtype, AaVsCfg& c)
     if (span * g.C > cap) return false;
     const int elems = span * g.C + slack;
     c.ve = (elems + E - 1) / E * E;
-    c.nt = std::min(kVsNT, (c.ve / E + 31) / 32 * 32);
+    c.nt = std::min(kVsMaxNT, (c.ve / E + 31) / 32 * 32);
     c.raw_row = std::max((elems * es + 15) / 16 + 2, (15 + elems * es + 4 * vs_words(es) + 15) / 16) * 16;
-    c.chunk = es == 1 ? 8 : 4;
     const int S = c.raw_row + (int)((g.src_pitch * es) & 15);
     const double f = (double)g.H / g.Ho, reach = 2.0 * (method == M_BILINEAR ? 1 : 2) * f + 20.0;
     const int64_t cols = (int64_t)((g.Wo + c.TW - 1) / c.TW) * g.planes;
@@ -143,24 +147,30 @@ bool aa_vs_config(const Geom& g, int method, int dtype, AaVsCfg& c)
     bool any = false;
     double best = 0.0;
     AaVsCfg fit = c;
-    for (int k : {3, 4, 8, 12, 16}) {   // blocks per SM (4 are resident)
-        const int64_t bands = std::max<int64_t>(1, k * (int64_t)sms / cols);
-        AaVsCfg t = c;
-        t.TH = (int)std::max<int64_t>(1, (g.Ho + bands - 1) / bands);
-        for (;; t.TH = (t.TH + 1) / 2) {
-            t.nr = aa_span_bound(t.TH, g.H, g.Ho, method);
-            t.smem = 3 * (size_t)vs_rows_bytes(t.chunk, S) + sizeof(float2) * (2 * (size_t)t.ve + (size_t)t.nr * t.NA) +
-                     sizeof(float) * (size_t)t.TW * t.KX + sizeof(int) * (2 * (size_t)t.TW + t.TH);
-            if (t.smem <= max_smem_per_block() || t.TH == 1) break;
-        }
-        if (t.smem > max_smem_per_block()) continue;
-        const double per_sm = std::ceil(cols * ((g.Ho + t.TH - 1) / t.TH) / sms);
-        const double resident = std::max(1.0, std::floor(224.0 * 1024 / (t.smem + 1024)));
-        const double cost = per_sm * (t.TH * f + reach) * std::max(1.0, 3.0 / std::min(resident, per_sm));
-        if (!any || cost < best) {
-            fit = t;
-            best = cost;
-            any = true;
+    c.chunk = es == 1 ? 8 : 4;
+    // Row weights as pairs (8 NA bytes a row), or where not even one output
+    // row's fit (bicubic from ~5500 source rows on) once, 4 NA bytes.
+    for (c.single = 0; c.single < 2 && !any; ++c.single) {
+        for (int k : {3, 4, 8, 12, 16}) {   // blocks per SM (4 are resident)
+            const int64_t bands = std::max<int64_t>(1, k * (int64_t)sms / cols);
+            AaVsCfg t = c;
+            t.TH = (int)std::max<int64_t>(1, (g.Ho + bands - 1) / bands);
+            for (;; t.TH = (t.TH + 1) / 2) {
+                t.nr = aa_span_bound(t.TH, g.H, g.Ho, method);
+                t.smem = 3 * (size_t)vs_rows_bytes(t.chunk, S) + sizeof(float2) * (2 * (size_t)t.ve + (size_t)(t.single ? t.chunk : t.nr) * t.NA) +
+                         (t.single ? sizeof(float) * (size_t)t.nr * t.NA : 0) +
+                         sizeof(float) * (size_t)t.TW * t.KX + sizeof(int) * (2 * (size_t)t.TW + t.TH);
+                if (t.smem <= max_smem_per_block() || t.TH == 1) break;
+            }
+            if (t.smem > max_smem_per_block()) continue;
+            const double per_sm = std::ceil(cols * ((g.Ho + t.TH - 1) / t.TH) / sms);
+            const double resident = std::max(1.0, std::floor(224.0 * 1024 / (t.smem + 1024)));
+            const double cost = per_sm * (t.TH * f + reach) * std::max(1.0, 3.0 / std::min(resident, per_sm));
+            if (!any || cost < best) {
+                fit = t;
+                best = cost;
+                any = true;
+            }
         }
     }
     if (any) c = fit;

@@ -151,9 +151,10 @@ struct AaWideCfg {
 // of a finished row (the widest tile footprint times the channels, rounded up
 // to a thread's); nr = the most source rows of a band of TH output rows;
 // chunk = rows per copy-ring slot; raw_row = bytes per raw ring row; aligned:
-// the source rows lie a whole number of a thread's elements apart.
+// the source rows lie a whole number of a thread's elements apart; single: the
+// row weights are kept once, not as pairs.
 struct AaVsCfg {
-    int KX, TW, TH, NA, ve, nr, chunk, raw_row, method, nt, aligned;
+    int KX, TW, TH, NA, ve, nr, chunk, raw_row, method, nt, aligned, single;
     size_t smem;
 };
 
