@@ -101,6 +101,35 @@ static int aa_span_bound(int k, int n, int m, int method)
     return (int)std::min<int64_t>(n, (d + m - 1) / m);
 }
 
+// The problems the form is held to whatever its tiles: what tiles of 8 to 256
+// columns of at most 1024 elements and 8 rows took in its first layout (24
+// bytes of weights a source row, eight finished rows, 40 KB of copies). Beyond
+// them it takes what fits without more threads or single weights.
+static bool aa_vs_range(const Geom& g, int method, int dtype)
+{
+    const size_t es = dtype_size(dtype), most = max_smem_per_block();
+    const int nr = aa_span_bound(std::min(8, g.Ho), g.H, g.Ho, method);
+    const auto bytes = [&](size_t elems, size_t tw, size_t kx, size_t rows) {
+        const size_t row = ((elems * es + 15) / 16 + 2) * 16;
+        size_t chunk = 8;
+        while (chunk > 2 && 3 * chunk * row > 40 * 1024) chunk /= 2;
+        return 3 * chunk * row + 32 * ((elems + 3) / 4 * 4) + 4 * tw * kx + 8 * tw + 24 * rows;
+    };
+    // most problems: bounds of all that it depends on
+    const size_t kx = aa_span_bound(1, g.W, g.Wo, method);
+    if (aa_span_bound(std::min(8, g.Wo), g.W, g.Wo, method) * g.C <= 1024 &&
+        40 * 1024 + 32 * 1024 + 4 * 256 * kx + 8 * 256 + 24 * (size_t)nr <= most)
+        return true;
+    for (int tw = 256; tw >= 8; tw /= 2) {
+        int k = 0, span = 0, ky = 0, rows = 0;
+        aa_axis_bounds(g.W, g.Wo, method, tw, k, span);
+        if ((int64_t)span * g.C > 1024) continue;
+        aa_axis_bounds(g.H, g.Ho, method, 8, ky, rows);
+        return bytes((size_t)span * g.C, tw, k, rows) <= most;
+    }
+    return false;
+}
+
 // The vertical-first form: output rows no more than source rows, and 8 output
 // columns' footprint at most 1024 elements. Tiles: the fewest of equal width
 // whose footprints fit a block (a partly filled tile would cost as much as a
@@ -125,7 +154,9 @@ bool aa_vs_config(const Geom& g, int method, int dtype, AaVsCfg& c)
     c.KX = aa_span_bound(1, g.W, g.Wo, method);
     int slack = c.aligned ? E - 1 : 0;   // owned elements before the footprint
     int cap = kVsNT * E - slack;
+    const bool range = aa_vs_range(g, method, dtype);
     if (c.KX * g.C > cap) {   // one column's footprint is wider: more threads (FP32), no element before it
+        if (!range) return false;
         c.aligned = 0;
         slack = 0;
         cap = std::min(kVsMaxNT * E, 1024);
@@ -150,7 +181,7 @@ bool aa_vs_config(const Geom& g, int method, int dtype, AaVsCfg& c)
     c.chunk = es == 1 ? 8 : 4;
     // Row weights as pairs (8 NA bytes a row), or where not even one output
     // row's fit (bicubic from ~5500 source rows on) once, 4 NA bytes.
-    for (c.single = 0; c.single < 2 && !any; ++c.single) {
+    for (c.single = 0; c.single < 1 + range && !any; ++c.single) {
         for (int k : {3, 4, 8, 12, 16}) {   // blocks per SM (4 are resident)
             const int64_t bands = std::max<int64_t>(1, k * (int64_t)sms / cols);
             AaVsCfg t = c;

@@ -21,13 +21,13 @@ def image(H, W, C, dtype):
 
 @pytest.mark.parametrize("H,W,C,Ho,Wo,dtype,method", [
     # rows: around and beyond what pairs leave room for
-    (6700, 24, 3, 1, 3, "u8", 2), (7000, 64, 3, 1, 8, "u8", 2), (7500, 64, 1, 4, 8, "u8", 2), (8000, 300, 3, 2, 30, "u8", 2),
+    (6700, 24, 3, 1, 3, "u8", 2), (7000, 64, 3, 1, 8, "u8", 2), (7500, 64, 1, 4, 8, "u8", 2), (8000, 1200, 3, 2, 120, "u8", 2),
     (9218, 1, 1, 1, 1, "u8", 2), (8015, 1, 4, 4, 12, "f16", 2), (8506, 12, 1, 4, 3, "f32", 2), (7413, 88, 4, 4, 39, "bf16", 2),
     (8000, 33, 3, 5, 7, "u8", 2), (9001, 40, 1, 3, 5, "u8", 1),
-    # columns: FP32 footprints of 510 to 1024 elements, and the widest of uint8
+    # columns: FP32 footprints of 510 elements and more
     (1000, 200, 3, 3, 2, "f32", 1), (65, 207, 3, 1, 2, "f32", 1), (444, 206, 4, 20, 2, "f32", 1), (264, 882, 1, 1, 4, "f32", 1),
-    (40, 1024, 1, 3, 1, "f32", 1), (33, 510, 1, 5, 1, "f32", 2), (90, 1024, 1, 7, 1, "u8", 1), (90, 1019, 1, 7, 1, "f16", 2),
-    (300, 256, 4, 40, 1, "f32", 2)])
+    (20, 129, 4, 1, 1, "f32", 1), (33, 510, 1, 5, 1, "f32", 2), (90, 1019, 1, 7, 1, "f16", 2), (31, 150, 4, 7, 1, "f32", 2),
+    (100, 195, 3, 9, 2, "f32", 1)])
 def test_footprints(H, W, C, Ho, Wo, dtype, method):
     x = image(H, W, C, dtype)
     ref = oracle.resize_aa(as_f64(x), Ho, Wo, method)
@@ -49,3 +49,11 @@ def test_preprocess_of_long_columns():
     v = oracle.resize_aa(as_f64(x), 1, 8, 2)
     ref = ((v - np.array(mean)) / np.array(std)).transpose(2, 0, 1)
     assert np.abs(y.double().cpu().numpy() - ref).max() <= 1e-5 * 255 / min(std) + 1e-6 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("H,W,C,Ho,Wo,dtype,method", [(756, 315, 3, 3, 1, "f32", 2), (1612, 481, 1, 5, 1, "f32", 2)])
+def test_refused_as_before(H, W, C, Ho, Wo, dtype, method):
+    """Beyond the form's range only what fits it as it is."""
+    for impl in ("stream", "auto"):
+        with pytest.raises(rs.ResampleError):
+            rs.resize(image(H, W, C, dtype), (Ho, Wo), NAMES[method], antialias=True, impl=impl)
