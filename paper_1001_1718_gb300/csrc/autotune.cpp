@@ -174,7 +174,7 @@ static bool default_choice(const Geom& g, int method, int dtype, const void* src
         for (int ch : {8, 4}) {
             const Tuned t{RS_IMPL_WINDOW, 1024, ch, 128, waves};
             if (!make_choice(g, method, dtype, src, t, k) || k.window.smem > (ch == 8 ? 56 : 100) * 1024) continue;
-            if (k.window.pat) k.window.waves = std::min(waves, win_raw_waves(out_bytes));
+            if (k.window.pat) k.window.waves = std::min(waves, win_raw_waves(g, k.window, out_bytes));
             return true;
         }
     }

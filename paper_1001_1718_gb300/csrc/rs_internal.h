@@ -214,7 +214,7 @@ bool win_raw_config(const Geom& g, int method, int dtype, int nt, int band_cap, 
 bool win_raw_default(const Geom& g, int method, int dtype, int nt, int band_cap, WinCfg& c, bool allow_x2 = true);
 int win_raw_threads(int Wo, int warp_px);
 int win_raw_block(const Geom& g, int warp_px);   // its threads per block for a problem
-int win_raw_waves(int64_t out_bytes);           // its default blocks per resident slot
+int win_raw_waves(const Geom& g, const WinCfg& c, int64_t out_bytes);   // its default blocks per resident slot
 cudaError_t launch_win_raw(const Geom& g, int method, const void* src, void* dst, WinCfg c, cudaStream_t st);
 // Whether the pre-process's output suits the form better than the FP32 form of
 // configuration fp32 (win_raw.cu).

@@ -143,8 +143,18 @@ int win_raw_block(const Geom& g, int warp_px)
 // x2, RGB 653 x 1148 bilinear, 9 MB: 5.7 us in one, 7.6 in two, and 6.6 on the
 // form on FP32 windows that this one replaced; grey 32 x 485 x 171 -> 1570 x
 // 553 bilinear, 28 MB: 26.0, 29.2 and 27.4). The two cross near 45 MB (exact
-// x2, 16 planes of 356 x 2900, 66 MB: 28.6 in one, 25.5 in two).
-int win_raw_waves(int64_t out_bytes) { return out_bytes <= (int64_t)32 << 20 ? 1 : 2; }
+// x2, 16 planes of 356 x 2900, 66 MB: 28.6 in one, 25.5 in two). Two also
+// where whole bands of many strips and planes fill one round of slots worse
+// (512 planes of 407 x 22 doubled, 18 MB: 40.1, in one 48.5).
+int win_raw_waves(const Geom& g, const WinCfg& c, int64_t out_bytes)
+{
+    if (out_bytes > (int64_t)32 << 20) return 2;
+    const int64_t strip = raw_strip(c.nt, false), units = ((int64_t)g.Wo + strip - 1) / strip * g.planes;
+    const int64_t by_regs = (c.pat == kRawX2 + 1 ? 5 : 4) * kWinThreads / c.nt, by_smem = 228 * 1024 / ((int64_t)c.smem + 1024);
+    const int64_t slots = num_sms() * std::max<int64_t>(1, std::min(by_regs, by_smem));
+    const auto filled = [&](int64_t n) { return (double)std::max<int64_t>(1, n / units) * units / n; };
+    return filled(slots) < 0.95 * std::min(1.0, filled(2 * slots)) ? 2 : 1;
+}
 
 bool win_raw_config(const Geom& g, int method, int dtype, int nt, int band_cap, WinCfg& c, bool allow_x2)
 {
@@ -213,7 +223,7 @@ static cudaError_t launch_raw(const Geom& g, void* func, int strip, const void* 
     if (c.band_h <= 0) {
         const int64_t resident = (int64_t)num_sms() * std::max(1, per_sm);
         const int64_t elems = (int64_t)g.Ho * g.Wo * g.C * g.planes;
-        const int waves = c.waves > 0 ? c.waves : win_raw_waves(elems * (int64_t)(no ? dtype_size(no->dtype) : 1));
+        const int waves = c.waves > 0 ? c.waves : win_raw_waves(g, c, elems * (int64_t)(no ? dtype_size(no->dtype) : 1));
         // at most `waves` blocks per resident slot: a partial extra wave would run alone
         const int64_t bands = std::max<int64_t>(1, resident * waves / (strips * g.planes));
         c.band_h = (int)std::min<int64_t>(c.band_cap, std::max<int64_t>(1, (g.Ho + bands - 1) / bands));
