@@ -119,7 +119,8 @@ bool win_config(const Geom& g, int method, int dtype, WinCfg& c, bool allow_x2)
     // a downscale's block spends most of its time staging rows, which idle
     // lanes share, and so does each of a few short rows' blocks: RGBA
     // pre-process of 29 x 67 doubled 3.4 us, in narrow blocks 3.9)
-    const bool narrow = allow_x2 && g.Wo >= g.W && (int64_t)g.Ho * g.planes > 2 * num_sms();
+    const int64_t wide = ((int64_t)g.Wo + kWinThreads * P - 1) / (kWinThreads * P) * g.Ho * g.planes;   // one-row blocks
+    const bool narrow = allow_x2 && g.Wo >= g.W && wide > 2 * num_sms();
     c.nt = narrow ? win_raw_threads(g.Wo, 32 * P) : kWinThreads;
     const int SP = c.nt * P;
     c.pat = 0;
