@@ -364,11 +364,12 @@ def _descs(srcs, dsts, methods) -> tuple:
 
 def _describe(srcs, dsts, methods) -> tuple:
     """The descriptors, their number, and whether an image's rows shrink more
-    than 16 times."""
+    than 24 times."""
     n = len(srcs)
     shrunk = False
     buf = bytearray(n * _DESC.size)
-    codes = [_code(METHODS, methods[k], "method") for k in range(n)]
+    known = METHODS.get
+    codes = [known(methods[k]) or _code(METHODS, methods[k], "method") for k in range(n)]
     at = 0
     for s, d, m in zip(srcs, dsts, codes):
         if s.dim() != 3 or d.dim() != 3:
@@ -379,7 +380,7 @@ def _describe(srcs, dsts, methods) -> tuple:
             raise ValueError("batched images need dense pixels (pitched rows are fine)")
         _DESC.pack_into(buf, at, s.data_ptr(), d.data_ptr(), H, W, C, Ho, Wo, m, sr, dr)
         at += _DESC.size
-        if W > 16 * Wo:
+        if W > 24 * Wo:
             shrunk = True
     return (B.RsImageDesc * n).from_buffer(buf), n, shrunk
 
@@ -410,8 +411,8 @@ def resize_batched(srcs: Sequence[torch.Tensor], sizes, methods, *, coord="asymm
     arr, n, shrunk = _describe(srcs, outs, methods)
     dt = _dtype(srcs[0])
     # The query refuses what the call refuses (it checks the descriptors again)
-    # and batches whose default tiles do not fit in shared memory: with rows of
-    # 1/16 and more they always do.
+    # and batches whose default tiles do not fit in shared memory (bicubic rows
+    # below about 1/27).
     nbytes = None if shrunk else _CALLS.get(("batch", n))
     if nbytes is None:
         nbytes = _batch_bytes(arr, n, dt)

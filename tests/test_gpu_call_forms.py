@@ -42,10 +42,10 @@ def test_batch_refusals_do_not_depend_on_earlier_batches():
 
 @pytest.mark.parametrize("C", [1, 2, 3, 4])
 @pytest.mark.parametrize("method", ["nearest", "bilinear", "bicubic"])
-def test_rows_of_a_sixteenth_always_fit(C, method):
+def test_rows_of_a_24th_always_fit(C, method):
     """The ratio down to which the query's answer is kept."""
     for Wo in (1, 7, 64, 600):
-        x = torch.zeros(9, 16 * Wo, C, dtype=torch.uint8, device="cuda")
+        x = torch.zeros(9, 24 * Wo, C, dtype=torch.uint8, device="cuda")
         y = torch.zeros(5, Wo, C, dtype=torch.uint8, device="cuda")
         assert rs.batched_workspace_bytes([x], [y], [method]) > 0
         rs.resize_batched([x], [(5, Wo)], [method], outs=[y])
