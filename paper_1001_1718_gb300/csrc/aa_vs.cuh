@@ -242,6 +242,30 @@ __device__ __forceinline__ void aa_vs_body(const Geom& g, const T* __restrict__ 
         p += S;
         yw += NA;
     };
+    auto add_rows = [&](int to) {   // source rows y .. to - 1
+        while (y < to) {
+            if (y == y_end) next_chunk();   // uniform
+            const int ys = min(to, y_end);
+            for (; y < ys; ++y) add_row();
+        }
+    };
+    // Sets 1 .. NA - 1 take in the tile's first rows before their own rows
+    // begin, with weight 0: nothing, unless a row holds an infinity or a NaN
+    // (further down a set's next row begins where its last one ended). So a
+    // float set is cleared where its first row begins.
+    if constexpr (ES > 1) {
+        #pragma unroll 1
+        for (int q = 1; q < min(NA, ni); ++q) {
+            int lo, hi;
+            aa_range(i0 + q, g.H, g.Ho, m, lo, hi);
+            add_rows(lo - r_lo);
+            #pragma unroll
+            for (int t = 1; t < NA; ++t)
+                if (t == q)
+                    #pragma unroll
+                    for (int k = 0; k < E / 2; ++k) acc[t][k] = make_float2(0.0f, 0.0f);
+        }
+    }
     for (int f0 = 0; f0 < ni; f0 += 4) {
         if (ni - f0 <= 2 && own) {   // no second pair: nothing to blend from it
             float4* v = reinterpret_cast<float4*>(V + cfg.ve + e0);
@@ -251,12 +275,7 @@ __device__ __forceinline__ void aa_vs_body(const Geom& g, const T* __restrict__ 
         #pragma unroll
         for (int u = 0; u < 4; ++u) {
             if (f0 + u < ni) {   // uniform
-                const int yh = YH[f0 + u];
-                while (y < yh) {
-                    if (y == y_end) next_chunk();   // uniform
-                    const int ys = min(yh, y_end);
-                    for (; y < ys; ++y) add_row();
-                }
+                add_rows(YH[f0 + u]);
                 float2 (&a)[E / 2] = acc[u % NA];
                 if (u & 1) {
                     if (own) {
