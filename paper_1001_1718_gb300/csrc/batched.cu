@@ -541,7 +541,7 @@ static constexpr int kBandItems = 4;   // items wanted per resident block slot (
 static int default_band(const rs_image_desc* d, int n)
 {
     int64_t rows = 0;   // strips x output rows
-    for (int k = 0; k < n; ++k) rows += (int64_t)((std::max(d[k].Wo, 1) + 495) / 496) * std::max(d[k].Ho, 1);
+    for (int k = 0; k < n; ++k) rows += ((int64_t)std::max(d[k].Wo, 1) + 495) / 496 * std::max(d[k].Ho, 1);   // (sizes not checked yet)
     const int64_t band = rows / ((int64_t)kBandItems * 4 * num_sms());
     return (int)std::min<int64_t>(kWinMaxBand, std::max<int64_t>(32, (band + 7) / 8 * 8));
 }

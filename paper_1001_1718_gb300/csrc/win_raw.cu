@@ -64,7 +64,8 @@ static void* raw_func_s(int st)
 template <int C, int PAT, typename TO>
 static void* norm_func_t(int st)
 {
-    if (st == RAW_WORDS) return (void*)&k_win_raw_norm<kRawKT, C, PAT, RAW_WORDS, TO>;
+    if constexpr (C == 3 && PAT == kRawX2 && sizeof(TO) == 4) return nullptr;   // win_raw_norm_ok
+    else if (st == RAW_WORDS) return (void*)&k_win_raw_norm<kRawKT, C, PAT, RAW_WORDS, TO>;
     if constexpr (PAT == 2 || PAT == 4) return (void*)&k_win_raw_norm<kRawKT, C, PAT, RAW_ANY, TO>;
     return nullptr;
 }
