@@ -296,10 +296,12 @@ typedef struct {
  * impl = RS_IMPL_AUTO: bilinear / bicubic images whose source footprint
  *   fits run as register-window items (bands of 32 to 256 output rows, by
  *   the batch's work; source rows staged 8 at a time, else 4), the rest as
- *   tiles; when
- *   rs_autotune_batched has tuned this batch (same sizes, methods, pitches,
- *   dtype, count and coord) its shape is used instead. An explicit tile_w /
- *   tile_h / threads tiles every image.
+ *   tiles; uint8 images of up to two source pixels per output pixel along x
+ *   are read in place, unless that adds six launches or more to a small
+ *   batch (of several channel counts); when rs_autotune_batched has tuned
+ *   this batch (same sizes, methods, pitches, dtype, count and coord) its
+ *   shape is used instead. An explicit tile_w / tile_h / threads tiles every
+ *   image.
  * impl = RS_IMPL_WINDOW: window items with band = tile_w output rows
  *   (1..256, 0 = 256) and chunk = tile_h staged rows (4..32, a multiple of
  *   the taps, 0 = 8 else 4);
@@ -359,7 +361,9 @@ rs_status rs_resize_batched_noalloc(const rs_image_desc* d, int n, rs_dtype dtyp
  * Replayable batch: the work list is uploaded once and the persistent launch
  * is recorded as a CUDA graph; each rs_batched_plan_launch replays it on a
  * stream. The plan refers to the descriptors' src / dst buffers and to
- * `workspace`, which must stay valid until rs_batched_plan_destroy.
+ * `workspace`, which must stay valid until rs_batched_plan_destroy. Every
+ * replay writes the workspace too (the classes' item counters): it belongs to
+ * one plan, whose replays run in order.
  */
 typedef struct rs_batched_plan rs_batched_plan;
 rs_status rs_batched_plan_create(const rs_image_desc* d, int n, rs_dtype dtype,

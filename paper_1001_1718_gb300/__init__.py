@@ -242,7 +242,7 @@ def resize_normalize(x: torch.Tensor, size: Sequence[int], method="bilinear", me
     (N, H, W, C) image, normalise every channel, (y - mean[c]) / std[c], and
     return it planar, (C, Ho, Wo) or (N, C, Ho, Wo), as FP16 / BF16 / FP32,
     in one pass (rs_resize_normalize). antialias=True stretches the filter
-    by the downscale factor (RS_FLAG_ANTIALIAS, at most 8 taps per axis)."""
+    by the downscale factor (RS_FLAG_ANTIALIAS)."""
     _require_cuda(x)
     if x.dtype != torch.uint8:
         raise ValueError("resize_normalize reads uint8 images")

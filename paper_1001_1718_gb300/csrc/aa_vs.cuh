@@ -17,21 +17,22 @@
 // the stretched kernel is NA output steps long, and output row i + NA starts
 // at or below row i's last tap). A per-row table holds the row's weight in
 // each set, row i in set i mod NA, 0 elsewhere, as the pair that a packed FMA
-// takes; where the pairs of a tile's rows do not fit in shared memory the table
-// holds the weights once and the pairs of one chunk at a time (single). The loop over output rows is
-// unrolled four times, so the sets are registers with fixed roles: row i is
-// complete where its taps end. Four complete rows go to shared memory as two
-// interleaved pairs, and between two barriers the block blends them with the
-// x taps (a thread per output column, two rows per packed FMA) and stores the
-// outputs. Sums run over the taps in ascending order, y first, then x.
+// takes; where the pairs of one output row do not fit in shared memory the
+// table holds the weights once and the pairs of one chunk at a time (single).
+// The loop over output rows is unrolled four times, so the sets are registers
+// with fixed roles: row i is complete where its taps end. Four complete rows
+// go to shared memory as two interleaved pairs, and between two barriers the
+// block blends them with the x taps (a thread per output column, two rows per
+// packed FMA) and stores the outputs. Sums run over the taps in ascending
+// order, y first, then x.
 //
 // What bounds it: instruction issue at 16 warps per SM (16 RGB 1080p frames to
 // 455 x 256, bilinear: 34 M warp instructions, about half the issue slots; 36
 // per source row and warp, a quarter of all in the blend, a tenth in a
 // block's start-up). The form it replaces (4 elements per thread read byte by
 // byte, sums in slots selected at run time, tiles of a power-of-two width)
-// issued 134 M. Measured: 177 -> 59 us; on the way, against 62-65: the words read by funnel
-// shifts at every pitch 70; five blocks of 96 registers per SM 67.
+// issued 134 M. Measured: 177 -> 59 us; on the way, against 62-65: the words
+// read by funnel shifts at every pitch 70; five blocks of 96 registers per SM 67.
 #pragma once
 
 #include <type_traits>

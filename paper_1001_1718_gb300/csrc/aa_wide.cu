@@ -180,7 +180,9 @@ bool aa_vs_config(const Geom& g, int method, int dtype, AaVsCfg& c)
     AaVsCfg fit = c;
     c.chunk = es == 1 ? 8 : 4;
     // Row weights as pairs (8 NA bytes a row), or where not even one output
-    // row's fit (bicubic from ~5500 source rows on) once, 4 NA bytes.
+    // row's fit (bicubic from ~5500 source rows on) once, 4 NA bytes: uint8 RGB
+    // 8000 x 1200 -> 2 x 120 1157 us (the form before: 1970). With more threads
+    // FP32 RGB 1000 x 200 -> 3 x 2 bilinear 103 us (278).
     for (c.single = 0; c.single < 1 + range && !any; ++c.single) {
         for (int k : {3, 4, 8, 12, 16}) {   // blocks per SM (4 are resident)
             const int64_t bands = std::max<int64_t>(1, k * (int64_t)sms / cols);

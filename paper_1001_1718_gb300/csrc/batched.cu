@@ -40,7 +40,7 @@ struct BatchImage {
     int H, W, Ho, Wo;
     int C, method, tiles_x, kind;          // tiles_x: items per row of items; kind 0 tile, 1 window, 2 many-tap, 3 window in place
     int tile_w, tile_h, sh_max, swe_max;   // kind 0: tiled-kernel tile
-    int chunk, band_h, swe, raw_row, band_cap, pos_cap, tab_off, raw_off;   // kind 1: window config
+    int chunk, band_h, swe, raw_row, band_cap, pos_cap, tab_off, raw_off;   // kinds 1 and 3: window config (swe: kind 1)
     int aa, strip;                         // antialias taps: the stretched method (0: point taps), window strip
     int KX, KY, TH, RG, fw, nr, s_off, pat;   // kind 3: pat (WinCfg); kind 2: many-tap antialias tiles (AaWideCfg)
 };
@@ -505,7 +505,8 @@ struct BatchLayout {
 };
 
 // Fills imgs_out (n entries) and start_out (n + kClasses prefix entries, then
-// kClasses zero item counters) grouped by class, with no allocation (scratch arrays are caller-provided, n each).
+// kClasses zero item counters) grouped by class, with no allocation (scratch
+// arrays are caller-provided, n each): batch_layout.
 // Tuning-cache key of a batch: GPU (model, CUDA runtime, SM count), dtype,
 // count, coordinate map and a hash of every descriptor's sizes, channels,
 // method and pitches.
@@ -636,9 +637,8 @@ static rs_status batch_layout(const rs_image_desc* d, int n, int dtype, const rs
         const int c = tmp_cls[k];
         imgs_out[L.first[c] + fill[c]++] = tmp_imgs[k];
     }
-    // Within a class, images with the costliest items first: block b takes
-    // items b, b + grid, ..., so neighbouring items of similar cost spread
-    // evenly over the blocks and the launch ends with the cheap ones.
+    // Within a class, images with the costliest items first: the blocks draw
+    // items in this order, so the launch ends with the cheap ones.
     for (int c = 0; c < kClasses; ++c) {
         BatchImage* first = imgs_out + L.first[c];
         std::sort(first, first + L.count[c], [](const BatchImage& a, const BatchImage& b) {

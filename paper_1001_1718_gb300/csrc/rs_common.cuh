@@ -296,6 +296,4 @@ __device__ __forceinline__ int aa_taps_n(int j, int n, int m, int method, float 
     return cnt;
 }
 
-// The work of one block: output tile (bx, by) of one plane (s, d: the
-// plane's first source / output element). Shared memory: cfg.smem bytes.
 }  // namespace rs

@@ -1,6 +1,7 @@
 // Register-window forward kernel for bilinear and bicubic resampling: one
-// block per (strip of kWinThreads * P output pixels, band of output rows,
-// plane); the block's work is win_body (win_body.cuh).
+// block of nt threads (at most kWinThreads; fewer where the rows are narrow) per
+// (strip of nt * P output pixels, band of output rows, plane); the block's work
+// is win_body (win_body.cuh).
 #include <algorithm>
 #include <climits>
 
